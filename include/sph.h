@@ -478,7 +478,7 @@ sph_status sph_backward(sph_ctx *ctx, const sph_grid *grid, const float *vel, co
  *   1 <= n <= SPH_SORT_STATIC_MAX_KEYS, else SPH_ERR_INVALID (also for NULL
  *   pointers); SPH_ERR_CUDA if a CUDA call fails.
  * Runs asynchronously on `stream` on the current device. Its scratch is a
- * fixed device array of about 12.6 MB inside the library, which every GPU
+ * fixed device array of about 13.7 MB inside the library, which every GPU
  * that uses it holds until the process exits. Every call looks up that
  * array's address in the current context (no allocation), so a context that
  * was reset and created again is handled. Set-up: under lazy module loading

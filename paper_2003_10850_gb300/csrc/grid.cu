@@ -62,7 +62,7 @@ template <typename P>
 __global__ void k_quantize(const P* __restrict__ pos, const float* __restrict__ mass, int n,
                            const long long* __restrict__ box_off, const BoxDesc* __restrict__ boxes,
                            int nb, int bb, uint4* __restrict__ xq, unsigned long long* __restrict__ keys,
-                           unsigned* __restrict__ vals, Counters* ctr) {
+                           Counters* ctr) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int lo = 0, hi = nb - 1;  // largest b with box_off[b] <= i
@@ -82,7 +82,6 @@ __global__ void k_quantize(const P* __restrict__ pos, const float* __restrict__ 
     if (bb) key = ((unsigned long long)lo << (63 - bb)) | (key >> bb);
     xq[i] = make_uint4(X, Y, Z, __float_as_uint(m));
     keys[i] = key;
-    vals[i] = (unsigned)i;
 }
 
 // ---------------------------------------------------------------------------
@@ -181,136 +180,248 @@ void scan_exclusive(const In* in, int n, uint32_t* out, uint32_t* tmp, cudaStrea
     *nl += 3;
 }
 template void scan_exclusive<uint8_t>(const uint8_t*, int, uint32_t*, uint32_t*, cudaStream_t, unsigned*);
-template void scan_exclusive<uint32_t>(const uint32_t*, int, uint32_t*, uint32_t*, cudaStream_t, unsigned*);
 
 // ---------------------------------------------------------------------------
-// a2: stable LSD radix sort of (64-bit key, 32-bit value), 8-bit digits
+// a2: stable LSD radix sort of (64-bit key, 32-bit index), 9-bit digits
 // ---------------------------------------------------------------------------
+//
+// One kernel counts every pass's digits, then one kernel per pass ranks and
+// moves the items: a tile of 4096 items finds where its digit runs start from
+// the digit totals and from the tiles before it, whose counts it reads as they
+// appear (each tile publishes its own counts first, then its running totals).
+// Tiles are numbered by a ticket, so a tile only ever waits for tiles that
+// already run. 63-bit keys take 7 passes of 9 bits: 9 launches in all.
+//
+// What bounds it: at 10M keys the 24 bytes per item and pass (HBM); below a
+// few hundred thousand the chain of passes, a few microseconds each. A
+// separate count, scan (three launches) and scatter per 8-bit pass, ranking
+// with four block barriers per 256 items, took 40 launches.
 
-constexpr int kRsT = 256, kRsIPT = 16, kRsTile = kRsT * kRsIPT;
+constexpr int kRsT = 512, kRsIPT = 8, kRsWarps = kRsT / 32;
+constexpr int kRsDig = 1 << kRsBits;
+static_assert(kRsTile == kRsT * kRsIPT && kRsDig == kRsT, "one digit per thread");
+constexpr int kRsSpin = 1 << 22;   // polls of a predecessor's word before giving up
+constexpr int kRsBack = 8;         // predecessors read at a time
 
-__global__ void k_rs_hist(const unsigned long long* __restrict__ keys, int n, int shift,
-                          unsigned* __restrict__ counts, int nblk) {
-    __shared__ unsigned hist[256];
-    hist[threadIdx.x] = 0;
+struct RsSmem {
+    unsigned long long key[kRsTile];
+    unsigned val[kRsTile];
+    unsigned short wcnt[kRsWarps][kRsDig];   // per warp: items of each digit so far; then the warps before
+    unsigned start[kRsDig];                  // first place of each digit's run in the tile
+    unsigned gbase[kRsDig];                  // global place of the run's first item - start
+    unsigned long long wsum[kRsWarps];
+    unsigned tile;
+};
+
+// The digit counts of every pass at once (keys are only permuted between passes).
+__global__ void __launch_bounds__(kRsT) k_rs_hist(const unsigned long long* __restrict__ keys, int n, int passes,
+                                                  unsigned* __restrict__ hist) {
+    __shared__ unsigned h[kRsMaxPass][kRsDig];
+    for (int p = 0; p < passes; ++p) h[p][threadIdx.x] = 0u;
     __syncthreads();
-    int base = blockIdx.x * kRsTile;
-#pragma unroll 4
-    for (int r = 0; r < kRsIPT; ++r) {
-        int k = base + r * kRsT + threadIdx.x;
-        if (k < n) atomicAdd(&hist[(unsigned)(keys[k] >> shift) & 255u], 1u);
+    for (long long base = (long long)blockIdx.x * kRsTile; base < n; base += (long long)gridDim.x * kRsTile) {
+        unsigned long long key[kRsIPT];
+#pragma unroll
+        for (int r = 0; r < kRsIPT; ++r) {
+            const long long k = base + r * kRsT + threadIdx.x;
+            key[r] = k < n ? keys[k] : 0ull;
+        }
+#pragma unroll
+        for (int r = 0; r < kRsIPT; ++r) {
+            if (base + r * kRsT + threadIdx.x < n)
+                for (int p = 0; p < passes; ++p)
+                    atomicAdd(&h[p][(unsigned)(key[r] >> (p * kRsBits)) & (kRsDig - 1u)], 1u);
+        }
     }
     __syncthreads();
-    counts[threadIdx.x * nblk + blockIdx.x] = hist[threadIdx.x];
+    for (int p = 0; p < passes; ++p) {
+        const unsigned c = h[p][threadIdx.x];
+        if (c) atomicAdd(&hist[p * kRsDig + threadIdx.x], c);
+    }
 }
 
-// Each block ranks its tile in rounds of 256 consecutive items; within a
-// round the rank of an item among equal digits is (items of earlier warps) +
-// (earlier lanes of its warp with the same digit), so the order of equal
-// digits is preserved (stable). The ranks place the tile's items in digit
-// order in shared memory (their tile indices); the items are then written
-// out in that order, so that consecutive threads write consecutive places of
-// a digit's run (coalesced) instead of one scattered place each.
-__global__ void __launch_bounds__(kRsT) k_rs_scatter(const unsigned long long* __restrict__ kin,
+// A word of the tiles' published counts: count, flag and the pass it belongs
+// to in one 64-bit word, so that no fence is needed and words of earlier
+// passes read as "not yet".
+__device__ __forceinline__ void rs_put(unsigned long long* p, unsigned tag, unsigned v) {
+    const unsigned long long w = ((unsigned long long)tag << 32) | v;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ unsigned long long rs_get(const unsigned long long* p) {
+    unsigned long long w;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+    return w;
+}
+
+// One pass. A warp ranks its 256 consecutive items in rounds of 32 (equal
+// digits in lane order, then round order: stable), the block adds the warps
+// before, and the items leave through shared memory in digit order, so that
+// consecutive threads write consecutive places of a digit's run. vin NULL: the
+// items' own indices. ctr (may be NULL) receives ST_TIMEOUT if a wait ran out;
+// every store stays inside [0, n) in any case.
+__global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* __restrict__ kin,
                                                      const unsigned* __restrict__ vin,
                                                      unsigned long long* __restrict__ kout,
-                                                     unsigned* __restrict__ vout, int n, int shift,
-                                                     const unsigned* __restrict__ offs,
-                                                     const unsigned* __restrict__ counts, int nblk) {
-    __shared__ unsigned short at[kRsTile];     // tile index of the item at each place of the tile
-    __shared__ unsigned start[256];             // first place of each digit's run in the tile
-    __shared__ unsigned run[256];               // places taken so far by each digit
-    __shared__ unsigned wcnt[kRsT / 32][256];
-    __shared__ unsigned wsum[kRsT / 32];
+                                                     unsigned* __restrict__ vout, int n, int pass,
+                                                     const unsigned* __restrict__ hist, unsigned* ticket,
+                                                     unsigned long long* status, Counters* ctr) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    RsSmem& sm = *reinterpret_cast<RsSmem*>(raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // exclusive scan of the tile's digit counts (one digit per thread)
+    const int shift = pass * kRsBits;
+    const unsigned agg = (unsigned)(pass + 1) * 2u, incl = agg + 1u;   // word tags: tile count, running total
+    if (tid == 0) sm.tile = atomicAdd(ticket, 1u);
     {
-        const unsigned c = counts[tid * nblk + blockIdx.x];
-        unsigned x = c;
+        unsigned* w = reinterpret_cast<unsigned*>(sm.wcnt[warp]);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        unsigned w0 = 0;
-        for (int w = 0; w < warp; ++w) w0 += wsum[w];
-        start[tid] = w0 + x - c;
-        run[tid] = w0 + x - c;
+        for (int k = 0; k < kRsDig / 64; ++k) w[k * 32 + lane] = 0u;
     }
-#pragma unroll
-    for (int w = 0; w < kRsT / 32; ++w) wcnt[w][tid] = 0;
+    const unsigned total = hist[tid];
     __syncthreads();
-    const int tile = blockIdx.x * kRsTile;
+    const int tile = (int)sm.tile;
+    const long long base = (long long)tile * kRsTile;
+    const int tn = (int)min((long long)kRsTile, n - base);
+    // places past n carry the last digit and the largest indices: they rank behind every item
+    unsigned long long key[kRsIPT];
+    unsigned val[kRsIPT], rank[kRsIPT];
+#pragma unroll
     for (int r = 0; r < kRsIPT; ++r) {
-        const int k = tile + r * kRsT + tid;
-        const bool valid = k < n;
-        const unsigned d = valid ? ((unsigned)(kin[k] >> shift) & 255u) : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const unsigned lt = peers & ((1u << lane) - 1u);
-        if (valid && lt == 0u) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        {
-            unsigned s = run[tid];
-#pragma unroll
-            for (int w = 0; w < kRsT / 32; ++w) {
-                const unsigned t = wcnt[w][tid];
-                wcnt[w][tid] = s;
-                s += t;
-            }
-            run[tid] = s;
-        }
-        __syncthreads();
-        if (valid) at[wcnt[warp][d] + __popc(lt)] = (unsigned short)(r * kRsT + tid);
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < kRsT / 32; ++w) wcnt[w][tid] = 0;
-        __syncthreads();
+        const int i = warp * (32 * kRsIPT) + r * 32 + lane;
+        key[r] = i < tn ? kin[base + i] : ~0ull;
+        val[r] = i < tn ? (vin ? vin[base + i] : (unsigned)(base + i)) : 0u;
     }
-    // write out in place order: place p of digit d goes to its run's global start
-    const int tn = min(kRsTile, n - tile);
-    for (int p = tid; p < tn; p += kRsT) {
-        const int i = tile + (int)at[p];
-        const unsigned long long key = kin[i];
-        const unsigned d = (unsigned)(key >> shift) & 255u;
-        const unsigned g = offs[d * nblk + blockIdx.x] + ((unsigned)p - start[d]);
-        kout[g] = key;
-        vout[g] = vin[i];
+#pragma unroll
+    for (int r = 0; r < kRsIPT; ++r) {
+        const int i = warp * (32 * kRsIPT) + r * 32 + lane;
+        const unsigned d = i < tn ? (unsigned)(key[r] >> shift) & (kRsDig - 1u) : kRsDig - 1u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int lead = __ffs(peers) - 1;
+        unsigned b = 0u;
+        if (lane == lead) {
+            b = sm.wcnt[warp][d];
+            sm.wcnt[warp][d] = (unsigned short)(b + __popc(peers));
+        }
+        b = __shfl_sync(0xffffffffu, b, lead);
+        rank[r] = b + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+    }
+    __syncthreads();
+    // thread tid serves digit tid from here on
+    unsigned cnt = 0u;
+#pragma unroll
+    for (int w = 0; w < kRsWarps; ++w) {
+        const unsigned c = sm.wcnt[w][tid];
+        sm.wcnt[w][tid] = (unsigned short)cnt;
+        cnt += c;
+    }
+    unsigned long long* mine = status + (size_t)tile * kRsDig + tid;
+    rs_put(mine, tile == 0 ? incl : agg, cnt);
+    // exclusive scans over the digits of the tile's counts (low word) and the totals (high word)
+    unsigned long long x = ((unsigned long long)total << 32) | cnt;
+    const unsigned long long own = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sm.wsum[warp] = x;
+    __syncthreads();
+    unsigned long long before = 0ull;
+#pragma unroll
+    for (int w = 0; w < kRsWarps; ++w) before += w < warp ? sm.wsum[w] : 0ull;
+    x += before - own;
+    sm.start[tid] = (unsigned)x;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRsIPT; ++r) {
+        const int i = warp * (32 * kRsIPT) + r * 32 + lane;
+        const unsigned d = i < tn ? (unsigned)(key[r] >> shift) & (kRsDig - 1u) : kRsDig - 1u;
+        const unsigned p = sm.start[d] + sm.wcnt[warp][d] + rank[r];
+        sm.key[p] = key[r];
+        sm.val[p] = val[r];
+    }
+    // the items of this digit in the tiles before: add their counts back to the
+    // nearest running total, several words in flight at a time
+    unsigned prefix = 0u;
+    int t = tile - 1, spins = 0;
+    while (t >= 0) {
+        unsigned long long w[kRsBack];
+#pragma unroll
+        for (int k = 0; k < kRsBack; ++k) w[k] = t - k >= 0 ? rs_get(status + (size_t)(t - k) * kRsDig + tid) : 0ull;
+        bool more = true;
+#pragma unroll
+        for (int k = 0; k < kRsBack; ++k) {
+            if (!more) continue;
+            const unsigned tag = (unsigned)(w[k] >> 32);
+            if (t < 0 || (tag != agg && tag != incl)) {
+                more = false;   // not published yet: read again from here
+            } else {
+                prefix += (unsigned)w[k];
+                t = tag == incl ? -1 : t - 1;
+                if (tag == incl) more = false;
+            }
+        }
+        if (t >= 0 && !more && ++spins > kRsSpin) {
+            if (ctr) atomicOr(&ctr->status, ST_TIMEOUT);
+            break;
+        }
+    }
+    if (tile > 0 && t < 0) rs_put(mine, incl, prefix + cnt);
+    sm.gbase[tid] = (unsigned)(x >> 32) + prefix - sm.start[tid];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRsIPT; ++r) {
+        const int p = r * kRsT + tid;
+        if (p < tn) {
+            const unsigned long long k = sm.key[p];
+            const unsigned g = sm.gbase[(unsigned)(k >> shift) & (kRsDig - 1u)] + (unsigned)p;
+            if (g < (unsigned)n) {
+                kout[g] = k;
+                vout[g] = sm.val[p];
+            }
+        }
     }
 }
 
-static void radix_sort(unsigned long long* keys, unsigned* vals, unsigned long long* keys2,
-                       unsigned* vals2, int n, int end_bit, unsigned* counts, unsigned* cscan,
-                       unsigned* tmp, cudaStream_t s, unsigned* nl) {
-    int nblk = (n + kRsTile - 1) / kRsTile;
-    unsigned long long *ka = keys, *kb = keys2;
-    unsigned *va = vals, *vb = vals2;
-    for (int shift = 0; shift < end_bit; shift += 8) {
-        k_rs_hist<<<nblk, kRsT, 0, s>>>(ka, n, shift, counts, nblk);
-        scan_exclusive<uint32_t>(counts, 256 * nblk, cscan, tmp, s, nl);
-        k_rs_scatter<<<nblk, kRsT, 0, s>>>(ka, va, kb, vb, n, shift, cscan, counts, nblk);
-        *nl += 2;
-        std::swap(ka, kb);
-        std::swap(va, vb);
+// Sorts keys of key_bits bits with their indices. kin is read by the first
+// pass only (and not written); the passes write (ka, va), (kb, vb), (ka, va),
+// ... in turn, so an odd number of passes ends in (ka, va). With an odd number
+// kin may be kb, with an even number kin may not be ka.
+cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsigned* va, unsigned long long* kb,
+                    unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, Counters* ctr,
+                    cudaStream_t s, unsigned* launches) {
+    const int passes = (key_bits + kRsBits - 1) / kRsBits;
+    const int tiles = (n + kRsTile - 1) / kRsTile;
+    unsigned* hist = reinterpret_cast<unsigned*>(work);
+    unsigned* ticket = hist + kRsMaxPass * kRsDig;
+    unsigned long long* status = reinterpret_cast<unsigned long long*>(work + kRsHead);
+    cudaError_t e = cudaFuncSetAttribute(k_rs_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RsSmem));
+    if (e) return e;
+    if ((e = cudaMemsetAsync(work, 0, rs_work_bytes(n), s))) return e;
+    k_rs_hist<<<std::min(tiles, 2 * sm_count), kRsT, 0, s>>>(kin, n, passes, hist);
+    if ((e = cudaGetLastError())) return e;
+    for (int p = 0; p < passes; ++p) {
+        k_rs_pass<<<tiles, kRsT, sizeof(RsSmem), s>>>(p == 0 ? kin : p & 1 ? ka : kb,
+                                                      p == 0 ? nullptr : p & 1 ? va : vb, p & 1 ? kb : ka,
+                                                      p & 1 ? vb : va, n, p, hist + p * kRsDig, ticket + p, status,
+                                                      ctr);
+        if ((e = cudaGetLastError())) return e;
     }
-    if (ka != keys) {
-        cudaMemcpyAsync(keys, ka, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(vals, va, sizeof(unsigned) * n, cudaMemcpyDeviceToDevice, s);
-    }
+    *launches += 1 + passes;
+    return cudaSuccess;
 }
 
 // ---------------------------------------------------------------------------
 // a3: gather into sorted order, hierarchy bounding boxes, h_max
 // ---------------------------------------------------------------------------
 
-__global__ void k_gather(const uint4* __restrict__ xq, const unsigned* __restrict__ sorted_vals, int n,
-                         uint4* __restrict__ posm, int32_t* __restrict__ perm, int32_t* __restrict__ rank) {
+__global__ void k_gather(const uint4* __restrict__ xq, int n, uint4* __restrict__ posm, int32_t* __restrict__ perm,
+                         int32_t* __restrict__ rank) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
-    int i = (int)sorted_vals[k];
+    int i = perm[k];
+    if ((unsigned)i >= (unsigned)n) perm[k] = i = k;   // only after a sort whose wait ran out (ST_TIMEOUT)
     posm[k] = xq[i];
-    perm[k] = i;
     rank[i] = k;
 }
 
@@ -405,11 +516,6 @@ __global__ void k_node_hmax(int lev, const BoxDesc* __restrict__ boxes, float* _
 // a6: active list
 // ---------------------------------------------------------------------------
 
-__global__ void k_iota(int32_t* a, int n) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) a[k] = k;
-}
-
 // all particles active: the identity list, and its length where the subset
 // path leaves the compacted count (scan[n])
 __global__ void k_iota_count(int32_t* a, int n, uint32_t* count) {
@@ -452,27 +558,31 @@ void grid_free(sph_grid* g) {
     if (!g) return;
     void* ptrs[] = {g->boxes, g->posm, g->xq, g->perm, g->rank, g->keys, g->node_lo, g->node_hi,
                     g->node_hmax, g->act, g->flag, g->scan, g->scan_tmp, g->list_a, g->list_b, g->st_lo, g->st_hi, g->list_n, g->d_off, g->d_L,
-                    g->k2, g->v1, g->v2, g->counts, g->cscan, g->node_c, g->node_e, g->posf,
+                    g->k2, g->v2, g->rs_work, g->node_c, g->node_e, g->posf,
                     g->fvel, g->fthermo, g->fposh, g->fvm, g->fbal, g->fcond, g->fvisc, g->node_m, g->box_rci, g->nbr, g->nbr_off, g->nbr_n, g->ext_n, g->ext, g->list_xh, g->list_st, g->fb_list, g->list_ep, g->mp_x, g->bw_ga, g->bw_xbar, g->bw_rd, g->bw_f, g->mp_j, g->den_left};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete g;
 }
 
-static void grid_fill(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s) {
+static cudaError_t grid_fill(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s) {
     sph_ctx* ctx = g->ctx;
     const int n = (int)g->n, nb = g->n_boxes;
     const int blocks = (n + 255) / 256;
+    // 7 passes: the sort starts from k2 and ends in (keys, perm)
+    unsigned long long* keys = (unsigned long long*)g->keys;
     if (f64)
         k_quantize<double><<<blocks, 256, 0, s>>>((const double*)pos, mass, n, g->d_off, g->boxes, nb, g->box_bits,
-                                                  g->xq, (unsigned long long*)g->keys, g->v1, ctx->counters);
+                                                  g->xq, g->k2, ctx->counters);
     else
         k_quantize<float><<<blocks, 256, 0, s>>>((const float*)pos, mass, n, g->d_off, g->boxes, nb, g->box_bits,
-                                                 g->xq, (unsigned long long*)g->keys, g->v1, ctx->counters);
+                                                 g->xq, g->k2, ctx->counters);
     ++ctx->launches;
-    radix_sort((unsigned long long*)g->keys, g->v1, g->k2, g->v2, n, 63, g->counts, g->cscan, g->scan_tmp, s,
-               &ctx->launches);
-    k_gather<<<blocks, 256, 0, s>>>(g->xq, g->v1, n, g->posm, g->perm, g->rank);
+    static_assert(((63 + kRsBits - 1) / kRsBits) % 2 == 1, "an odd number of passes ends in (keys, perm)");
+    const cudaError_t e = rs_sort(g->k2, keys, (unsigned*)g->perm, g->k2, g->v2, n, 63, g->rs_work, ctx->sm_count,
+                                  ctx->counters, s, &ctx->launches);
+    if (e) return e;
+    k_gather<<<blocks, 256, 0, s>>>(g->xq, n, g->posm, g->perm, g->rank);
     dim3 lg((g->max_leaves + 127) / 128, nb);
     k_leaf_bbox<<<lg, 128, 0, s>>>(g->posm, g->boxes, g->node_lo, g->node_hi, g->node_c, g->node_e, g->posf);
     ctx->launches += 2;
@@ -481,6 +591,7 @@ static void grid_fill(sph_grid* g, const void* pos, int f64, const float* mass, 
         k_node_bbox<<<ng, 128, 0, s>>>(lev, g->boxes, g->node_lo, g->node_hi, g->node_c, g->node_e);
         ++ctx->launches;
     }
+    return cudaGetLastError();
 }
 
 sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass, bool lists, const int64_t* offs,
@@ -532,9 +643,7 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
     g->max_leaves = maxleaf;
     g->max_lev = maxlev;
 
-    const int nblk = (n + kRsTile - 1) / kRsTile;
-    const int scan_words = 256 * nblk + 1;
-    const int tmp_words = std::max(n, scan_words) / kScanTile + 4;
+    const int tmp_words = n / kScanTile + 4;
     GRID_CHECK(cudaMalloc(&g->boxes, sizeof(BoxDesc) * nb));
     GRID_CHECK(cudaMemcpyAsync(g->boxes, g->boxes_h.data(), sizeof(BoxDesc) * nb, cudaMemcpyHostToDevice, s));
     GRID_CHECK(cudaMalloc(&g->d_off, sizeof(long long) * (nb + 1)));
@@ -605,12 +714,9 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
     GRID_CHECK(cudaMalloc(&g->st_hi, sizeof(float) * n));
     GRID_CHECK(cudaMalloc(&g->list_n, sizeof(int) * 2));
     GRID_CHECK(cudaMalloc(&g->k2, sizeof(unsigned long long) * n));
-    GRID_CHECK(cudaMalloc(&g->v1, sizeof(unsigned) * n));
     GRID_CHECK(cudaMalloc(&g->v2, sizeof(unsigned) * n));
-    GRID_CHECK(cudaMalloc(&g->counts, sizeof(unsigned) * scan_words));
-    GRID_CHECK(cudaMalloc(&g->cscan, sizeof(unsigned) * (scan_words + 1)));
-    grid_fill(g, pos, f64, mass, s);
-    GRID_CHECK(cudaGetLastError());
+    GRID_CHECK(cudaMalloc(&g->rs_work, rs_work_bytes(n)));
+    GRID_CHECK(grid_fill(g, pos, f64, mass, s));
     GRID_CHECK(cudaStreamSynchronize(s));
     *out = g;
     return SPH_OK;
@@ -618,8 +724,7 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
 
 sph_status grid_update(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s) {
     g->lists_rec = false;   // the particles may have moved: recorded neighbour lists are stale
-    grid_fill(g, pos, f64, mass, s);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = grid_fill(g, pos, f64, mass, s);
     if (e) {
         g->ctx->err = std::string("CUDA error in grid update: ") + cudaGetErrorString(e);
         return SPH_ERR_CUDA;

@@ -71,10 +71,8 @@ struct sph_grid {
     long long* d_off = nullptr;
     double* d_L = nullptr;
     unsigned long long* k2 = nullptr;
-    unsigned* v1 = nullptr;
     unsigned* v2 = nullptr;
-    unsigned* counts = nullptr;
-    unsigned* cscan = nullptr;
+    unsigned char* rs_work = nullptr;      // rs_sort's counts (rs_work_bytes(n))
     int32_t* mp_j = nullptr;               // density, member-parallel path: near-list indices per persistent warp
     int32_t* den_left = nullptr;           // density: particles left to the one-particle kernel (n)
     // neighbour lists recorded by an all-active density call on the default path and
@@ -137,6 +135,17 @@ void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStrea
 // exclusive scan of n values into out[0..n] (out[n] = total); tmp >= n/4096+2 words
 template <typename In>
 void scan_exclusive(const In* in, int n, uint32_t* out, uint32_t* tmp, cudaStream_t s, unsigned* launches);
+// stable radix sort of (key, index) pairs, see grid.cu; work: rs_work_bytes(n) bytes, 16-byte aligned
+constexpr int kRsBits = 9;          // bits per pass
+constexpr int kRsTile = 4096;       // items per block
+constexpr int kRsMaxPass = 8;
+constexpr size_t kRsHead = sizeof(unsigned) * (kRsMaxPass * (1 << kRsBits) + 2 * kRsMaxPass);   // digit counts, tickets
+constexpr size_t rs_work_bytes(int64_t n) {
+    return kRsHead + sizeof(unsigned long long) * (1 << kRsBits) * (size_t)((n + kRsTile - 1) / kRsTile);
+}
+cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsigned* va, unsigned long long* kb,
+                    unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, Counters* ctr,
+                    cudaStream_t s, unsigned* launches);
 // SPH_TIME_KERNELS support: event pair around one kernel launch
 cudaEvent_t timing_event(sph_ctx* ctx);
 

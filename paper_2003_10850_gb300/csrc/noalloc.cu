@@ -11,30 +11,16 @@
 // loads the library holds until the process exits.
 #include "internal.cuh"
 
-namespace sph {
-// kernels of the grid build (grid.cu), reused unchanged
-__global__ void k_rs_hist(const unsigned long long* keys, int n, int shift, unsigned* counts, int nblk);
-__global__ void k_rs_scatter(const unsigned long long* kin, const unsigned* vin, unsigned long long* kout,
-                             unsigned* vout, int n, int shift, const unsigned* offs, const unsigned* counts,
-                             int nblk);
-__global__ void k_iota(int32_t* a, int n);
-}  // namespace sph
-
 namespace {
 
 constexpr int kMaxKeys = SPH_SORT_STATIC_MAX_KEYS;
-constexpr int kTile = 4096;                            // keys per block of a radix pass
-constexpr int kBlocks = (kMaxKeys + kTile - 1) / kTile;
-constexpr int kCountWords = 256 * kBlocks + 1;
 
 // byte offsets of the sub-buffers (each 256-byte aligned)
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t kOffKeys = 0;
 constexpr size_t kOffVals = align256(kOffKeys + sizeof(unsigned long long) * kMaxKeys);
-constexpr size_t kOffCounts = align256(kOffVals + sizeof(unsigned) * kMaxKeys);
-constexpr size_t kOffScan = align256(kOffCounts + sizeof(unsigned) * kCountWords);
-constexpr size_t kOffTmp = align256(kOffScan + sizeof(unsigned) * (kCountWords + 1));
-constexpr size_t kScratchBytes = align256(kOffTmp + sizeof(unsigned) * 64);
+constexpr size_t kOffWork = align256(kOffVals + sizeof(unsigned) * kMaxKeys);
+constexpr size_t kScratchBytes = align256(kOffWork + sph::rs_work_bytes(kMaxKeys));
 
 // The scratch itself. Host code must not use this name as a device address:
 // on the host it names a stand-in object; the device address comes from
@@ -70,34 +56,22 @@ extern "C" sph_status sph_sort_keys_static(const uint64_t* keys, int64_t n, uint
     if (st != SPH_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     const int nn = (int)n;
-    const int nblk = (nn + kTile - 1) / kTile;
     unsigned long long* kb = reinterpret_cast<unsigned long long*>(base + kOffKeys);
     unsigned* vb = reinterpret_cast<unsigned*>(base + kOffVals);
-    unsigned* counts = reinterpret_cast<unsigned*>(base + kOffCounts);
-    unsigned* cscan = reinterpret_cast<unsigned*>(base + kOffScan);
-    unsigned* tmp = reinterpret_cast<unsigned*>(base + kOffTmp);
-    // Every scratch word a pass reads is written earlier in the same pass
-    // (histograms, their scan, the scattered keys), so nothing left over from
-    // an earlier call is read and nothing needs clearing.
-    unsigned long long* ka = reinterpret_cast<unsigned long long*>(sorted_keys);
-    unsigned* va = reinterpret_cast<unsigned*>(perm);
-    if (cudaMemcpyAsync(ka, keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return SPH_ERR_CUDA;
-    sph::k_iota<<<(nn + 255) / 256, 256, 0, s>>>(perm, nn);
-    if (cudaGetLastError() != cudaSuccess) return SPH_ERR_CUDA;
+    // Every scratch word the sort reads is cleared or written earlier in the
+    // same call, so nothing left over from an earlier call is read. 64 key bits
+    // take 8 passes, (kb, vb) first: an even count, so the result ends in the
+    // caller's buffers. Each launch is checked as it is queued, and the first
+    // failure stops the sort.
+    static_assert(((64 + sph::kRsBits - 1) / sph::kRsBits) == sph::kRsMaxPass, "an even number of passes");
     unsigned launches = 0;
-    // 8 passes of 8 bits over all 64 key bits: an even count, so the result
-    // ends in the caller's buffers. Each launch is checked as it is queued, and
-    // the first failure stops the sort.
-    for (int shift = 0; shift < 64; shift += 8) {
-        sph::k_rs_hist<<<nblk, 256, 0, s>>>(ka, nn, shift, counts, nblk);
-        if (cudaGetLastError() != cudaSuccess) return SPH_ERR_CUDA;
-        sph::scan_exclusive<uint32_t>(counts, 256 * nblk, cscan, tmp, s, &launches);
-        if (cudaGetLastError() != cudaSuccess) return SPH_ERR_CUDA;
-        sph::k_rs_scatter<<<nblk, 256, 0, s>>>(ka, va, kb, vb, nn, shift, cscan, counts, nblk);
-        if (cudaGetLastError() != cudaSuccess) return SPH_ERR_CUDA;
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return SPH_ERR_CUDA;
+    if (sph::rs_sort(reinterpret_cast<const unsigned long long*>(keys), kb, vb,
+                     reinterpret_cast<unsigned long long*>(sorted_keys), reinterpret_cast<unsigned*>(perm), nn, 64,
+                     base + kOffWork, sms, nullptr, s, &launches) != cudaSuccess)
+        return SPH_ERR_CUDA;
     return SPH_OK;
 }
