@@ -96,7 +96,7 @@ struct sph_grid {
     // adjoint scratch (allocated by the first sph_backward on the grid)
     float4* bw_ga = nullptr;
     float4* bw_xbar = nullptr;
-    float2* bw_rd = nullptr;
+    float4* bw_rd = nullptr;
     float* bw_f = nullptr;
 };
 
