@@ -290,19 +290,30 @@ __global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* _
         key[r] = i < tn ? kin[base + i] : ~0ull;
         val[r] = i < tn ? (vin ? vin[base + i] : (unsigned)(base + i)) : 0u;
     }
+    // the lanes of each round with the same digit, bit by bit (independent of one
+    // another, unlike the running counts that follow)
+    unsigned peers[kRsIPT];
 #pragma unroll
     for (int r = 0; r < kRsIPT; ++r) {
         const int i = warp * (32 * kRsIPT) + r * 32 + lane;
         const unsigned d = i < tn ? (unsigned)(key[r] >> shift) & (kRsDig - 1u) : kRsDig - 1u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const int lead = __ffs(peers) - 1;
-        unsigned b = 0u;
-        if (lane == lead) {
-            b = sm.wcnt[warp][d];
-            sm.wcnt[warp][d] = (unsigned short)(b + __popc(peers));
+        unsigned m = 0xffffffffu;
+#pragma unroll
+        for (int b = 0; b < kRsBits; ++b) {
+            const bool one = (d >> b) & 1u;
+            const unsigned v = __ballot_sync(0xffffffffu, one);
+            m &= one ? v : ~v;
         }
-        b = __shfl_sync(0xffffffffu, b, lead);
-        rank[r] = b + __popc(peers & ((1u << lane) - 1u));
+        peers[r] = m;
+        rank[r] = d;
+    }
+#pragma unroll
+    for (int r = 0; r < kRsIPT; ++r) {
+        const unsigned d = rank[r], b = sm.wcnt[warp][d];
+        const unsigned before = __popc(peers[r] & ((1u << lane) - 1u));
+        __syncwarp();   // every lane has read its digit's count
+        if (before == 0u) sm.wcnt[warp][d] = (unsigned short)(b + __popc(peers[r]));
+        rank[r] = b + before;
         __syncwarp();
     }
     __syncthreads();
