@@ -51,11 +51,12 @@ sph_status check_params(sph_ctx* ctx, const sph_params* p) {
 // warp-per-particle kernels run (member-parallel for groups, one particle per
 // warp for the rest): on the 10M clustered time bins they are the fastest at
 // every active fraction measured (100, 10, 1 and 0.1 %). SPH_FP64 selects the
-// per-thread walks in double.
-enum class Path { Plain, Wpp, Thread };
+// one-particle-per-warp kernels in double, whatever the path flag.
+enum class Path { Plain, Wpp, Thread, F64 };
 Path pick_path(int flags) {
     if (flags & SPH_PLAIN_FP32) return Path::Plain;
-    if (flags & (SPH_PER_THREAD_WALK | SPH_DENSITY_BUFFERED | SPH_FP64)) return Path::Thread;
+    if (flags & SPH_FP64) return Path::F64;
+    if (flags & (SPH_PER_THREAD_WALK | SPH_DENSITY_BUFFERED)) return Path::Thread;
     return Path::Wpp;
 }
 
@@ -226,7 +227,6 @@ static sph_status density_call(sph_ctx* ctx, const sph_grid* grid, float* h, con
     a.max_iter = params->max_iter;
     a.fixed_h = (params->flags & SPH_FIXED_H) ? 1 : 0;
     a.guess_h = (params->flags & SPH_H_GUESS) ? 1 : 0;
-    a.fp64 = (params->flags & SPH_FP64) ? 1 : 0;
     a.blocks_per_sm = params->blocks_per_sm;
     a.walk_radius = params->walk_radius;
     a.group_span = params->group_size;
@@ -240,6 +240,7 @@ static sph_status density_call(sph_ctx* ctx, const sph_grid* grid, float* h, con
     g->lists_rec = false;   // set again by a call that records neighbour lists
     cudaError_t e = path == Path::Plain ? run_density_plain(ctx, a, na, s)
                     : path == Path::Wpp ? launch_density_wpp(ctx, a, na, s)
+                    : path == Path::F64 ? launch_density_f64(ctx, a, na, s)
                                         : launch_density_tpp(ctx, a, na, s);
     if (!e) e = cudaGetLastError();
     if (e) return cuda_fail(ctx, e, "sph_density");
@@ -298,7 +299,6 @@ static sph_status force_call(sph_ctx* ctx, const sph_grid* grid, const float* ve
     a.hash = reinterpret_cast<unsigned long long*>(hash);
     a.alpha = params->alpha_visc;
     a.gamma = params->gamma;
-    a.fp64 = (params->flags & SPH_FP64) ? 1 : 0;
     a.blocks_per_sm = params->blocks_per_sm;
     a.group_span = params->group_size;
     a.time_kernels = (params->flags & SPH_TIME_KERNELS) ? 1 : 0;
@@ -309,6 +309,7 @@ static sph_status force_call(sph_ctx* ctx, const sph_grid* grid, const float* ve
     a.alpha_v = alpha_v;
     cudaError_t e = path == Path::Plain ? launch_force_plain(ctx, a, na, s)
                     : path == Path::Wpp ? launch_force_wpp(ctx, a, na, s)
+                    : path == Path::F64 ? launch_force_f64(ctx, a, na, s)
                                         : launch_force_tpp(ctx, a, na, s);
     if (!e) e = cudaGetLastError();
     if (e) return cuda_fail(ctx, e, "sph_hydro_force");

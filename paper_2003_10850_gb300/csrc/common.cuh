@@ -147,4 +147,38 @@ __device__ __forceinline__ bool exact_pred(unsigned long long D2, double HH) {
     return __ull2double_rn(D2) < HH;
 }
 
+// One bracketed step of the smoothing-length solve. f = N - N_t arrives in
+// FP64 (from the compensated FP32 sums); the bracket and the new h are kept in
+// FP64, while the Newton step on N^(1/3) - N_t^(1/3) is formed in FP32 (it is
+// a correction, and FP64 cbrt/division would cost ~60 FP32 slots each on this
+// part). Returns false when h cannot move (converged to the float grid or an
+// error bit was set).
+__device__ __forceinline__ bool h_update(float& h, double f, float N, float dN, float n_target, double cap,
+                                         double& blo, double& bhi, float& dold, unsigned& st) {
+    if (f < 0) blo = h; else bhi = h;
+    float step = dN > 0.f ? 3.f * N * (1.f - cbrtf(n_target / N)) / dN : NAN;
+    double hn = (double)h - (double)step;
+    if (isinf(bhi)) {
+        if ((double)h >= cap) {
+            st |= ST_H_TOO_LARGE;
+            return false;
+        }
+        if (!(hn > (double)h)) hn = 2.0 * (double)h;
+        hn = fmin(hn, fmin(cap, 8.0 * (double)h));
+    } else if (!(hn > blo && hn < bhi) || !(fabsf(step) <= 0.5f * dold)) {
+        // outside the bracket, or not converging fast (the step did not halve):
+        // bisect (the safeguard of Newton-Raphson with bracketing)
+        hn = 0.5 * (blo + bhi);
+    }
+    dold = fabsf((float)(hn - (double)h));
+    float hf = (float)hn;
+    if (!(hf > (float)blo) || (!isinf(bhi) && !(hf < (float)bhi))) {
+        const float mid = (float)(0.5 * (blo + bhi));
+        hf = (mid > (float)blo && mid < (float)bhi) ? mid : h;
+    }
+    if (hf == h) return false;  // the bracket is one float wide: h is the best float
+    h = hf;
+    return true;
+}
+
 }  // namespace sph

@@ -161,7 +161,6 @@ struct DensityLaunch {
     double n_target, n_tol;
     int max_iter;
     int fixed_h, guess_h;
-    int fp64;
     int blocks_per_sm;
     double walk_radius;   // 0: default
     int group_span = 0;   // sorted particles a group stays within (power of two; 0: default)
@@ -191,7 +190,6 @@ struct ForceLaunch {
     float* vsig;
     unsigned long long* hash;
     double alpha, gamma;
-    int fp64;
     int blocks_per_sm;
     int group_span = 0;   // as DensityLaunch
     int time_kernels;
@@ -237,6 +235,10 @@ cudaError_t launch_gravity(sph_ctx* ctx, const GravityLaunch& L, int64_t n_activ
 // wpp_density.cu, wpp_force.cu (one warp per particle)
 cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_active, cudaStream_t s);
 cudaError_t launch_force_wpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_active, cudaStream_t s);
+
+// f64.cu (SPH_FP64)
+cudaError_t launch_density_f64(sph_ctx* ctx, const DensityLaunch& a, int64_t n_active, cudaStream_t s);
+cudaError_t launch_force_f64(sph_ctx* ctx, const ForceLaunch& a, int64_t n_active, cudaStream_t s);
 
 // tpp.cu (per-thread walks)
 // list_xh / h_changed (optional): set *h_changed if some h differs from the h in list_xh;

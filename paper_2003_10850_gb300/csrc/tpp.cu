@@ -1,6 +1,6 @@
-// tpp.cu -- thread-per-particle density and force kernels (SPH_PER_THREAD_WALK,
-// and SPH_FP64 for the plain method in double; the default path is the
-// warp-per-group kernels of wpp_density.cu and wpp_force.cu), and the force
+// tpp.cu -- thread-per-particle density and force kernels (SPH_PER_THREAD_WALK;
+// the default path is the warp-per-group kernels of wpp_density.cu and
+// wpp_force.cu, SPH_FP64 runs the kernels of f64.cu), and the force
 // pass's per-particle packing (k_force_pack) that every force path reads.
 //
 // One thread per active particle, consecutive threads on Morton-consecutive
@@ -17,9 +17,7 @@
 //   * the neighbour predicate is exact ((double)D2 < H^2 on integer
 //     coordinates) inside a thin band around the FP32 radius test;
 //   * force candidates are read from packed per-call float4 records.
-// T = double runs the same walk with FP64 pair arithmetic on exact integer
-// separations.
-#include <type_traits>
+#include <algorithm>
 
 #include "internal.cuh"
 
@@ -28,16 +26,7 @@ namespace sph {
 constexpr int kTppThreads = 128;
 constexpr int kTppStack = 96;   // depth-first: <= 7 pending siblings per level + 1
 
-template <typename T>
-struct TBand;
-template <>
-struct TBand<float> {
-    static constexpr float rel = 9.5367431640625e-07f;  // 2^-20
-};
-template <>
-struct TBand<double> {
-    static constexpr double rel = 1.7763568394002505e-15;  // 2^-49
-};
+constexpr float kTppBand = 9.5367431640625e-07f;  // 2^-20
 
 __device__ __forceinline__ int tpp_box_of(const BoxDesc* boxes, int nb, long long p) {
     int lo = 0, hi = nb - 1;
@@ -61,46 +50,7 @@ __device__ __forceinline__ bool tpp_node_near(uint4 c, float4 e, uint4 X, float 
     return gx * gx + gy * gy + gz * gz < Rt * Rt;
 }
 
-template <typename T>
-__device__ __forceinline__ T tpp_sqrt(T x) {
-    if constexpr (std::is_same<T, float>::value) return x > 0.f ? x * rsqrtf(x) : 0.f;
-    else return sqrt(x);
-}
-
-
-// One bracketed step of the smoothing-length solve. f = N - N_t arrives in
-// FP64 (from the compensated FP32 sums); the bracket and the new h are kept in
-// FP64, while the Newton step on N^(1/3) - N_t^(1/3) is formed in FP32 (it is
-// a correction, and FP64 cbrt/division would cost ~60 FP32 slots each on this
-// part). Returns false when h cannot move (converged to the float grid or an
-// error bit was set).
-__device__ __forceinline__ bool h_update(float& h, double f, float N, float dN, float n_target, double cap,
-                                         double& blo, double& bhi, float& dold, unsigned& st) {
-    if (f < 0) blo = h; else bhi = h;
-    float step = dN > 0.f ? 3.f * N * (1.f - cbrtf(n_target / N)) / dN : NAN;
-    double hn = (double)h - (double)step;
-    if (isinf(bhi)) {
-        if ((double)h >= cap) {
-            st |= ST_H_TOO_LARGE;
-            return false;
-        }
-        if (!(hn > (double)h)) hn = 2.0 * (double)h;
-        hn = fmin(hn, fmin(cap, 8.0 * (double)h));
-    } else if (!(hn > blo && hn < bhi) || !(fabsf(step) <= 0.5f * dold)) {
-        // outside the bracket, or not converging fast (the step did not halve):
-        // bisect (the safeguard of Newton-Raphson with bracketing)
-        hn = 0.5 * (blo + bhi);
-    }
-    dold = fabsf((float)(hn - (double)h));
-    float hf = (float)hn;
-    if (!(hf > (float)blo) || (!isinf(bhi) && !(hf < (float)bhi))) {
-        const float mid = (float)(0.5 * (blo + bhi));
-        hf = (mid > (float)blo && mid < (float)bhi) ? mid : h;
-    }
-    if (hf == h) return false;  // the bracket is one float wide: h is the best float
-    h = hf;
-    return true;
-}
+__device__ __forceinline__ float tpp_sqrt(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
 
 // ---------------------------------------------------------------------------
 // Density
@@ -131,21 +81,19 @@ struct TppDensArgs {
     Counters* ctr;
 };
 
-template <typename T>
 struct TppDSums {
-    T sw, cw, sdw, cdw, smw, cmw, smdw, cmdw;
+    float sw, cw, sdw, cdw, smw, cmw, smdw, cmdw;
     int nn;
     unsigned long long hs, tests;
 };
 
-template <typename T, bool HASH>
+template <bool HASH>
 __device__ __forceinline__ void tpp_density_walk(const TppDensArgs& a, const BoxDesc& B, int p, uint4 Xi,
-                                                 float h, TppDSums<T>& S) {
+                                                 float h, TppDSums& S) {
     double HH = -1.0;  // (h 2^32/L)^2, formed on the first band pair only
     const double s = ldexp(B.L, -32);
     const float sf = (float)s;
-    const T sT = (T)s;
-    const T hT = (T)h, hinv = T(1) / hT;
+    const float hinv = 1.f / h;
     int stack[kTppStack];
     int sp = 0;
     stack[sp++] = B.nlev == 1 ? 0 : (B.nlev - 1) << 27;
@@ -165,28 +113,28 @@ __device__ __forceinline__ void tpp_density_walk(const TppDensArgs& a, const Box
         const int nd = B.lvl_off[0] + t;
         const uint4 C = a.node_c[nd];
         const float4 E = a.node_e[nd];
-        const T ox = (T)(int)(C.x - Xi.x) * sT, oy = (T)(int)(C.y - Xi.y) * sT, oz = (T)(int)(C.z - Xi.z) * sT;
+        const float ox = (float)(int)(C.x - Xi.x) * sf, oy = (float)(int)(C.y - Xi.y) * sf, oz = (float)(int)(C.z - Xi.z) * sf;
         // rounding bound of r for pairs in this leaf, and the predicate band
-        const T eL = TBand<T>::rel * (T(4) * (T)(E.x + E.y + E.z) + T(2) * (fabs(ox) + fabs(oy) + fabs(oz)) + T(2) * hT);
-        const T lo2 = hT > eL ? (hT - eL) * (hT - eL) * (T(1) - T(4) * TBand<T>::rel) : T(0);
-        const T hi2 = (hT + eL) * (hT + eL) * (T(1) + T(4) * TBand<T>::rel);
+        const float eL = kTppBand * (4.f * (E.x + E.y + E.z) + 2.f * (fabsf(ox) + fabsf(oy) + fabsf(oz)) + 2.f * h);
+        const float lo2 = h > eL ? (h - eL) * (h - eL) * (1.f - 4.f * kTppBand) : 0.f;
+        const float hi2 = (h + eL) * (h + eL) * (1.f + 4.f * kTppBand);
         const long long q0 = B.off + (long long)t * kLeaf, q1 = min(q0 + kLeaf, pend);
         // A leaf straddling a large Morton jump can be wider than half the box;
         // then centre offset + in-leaf offset is not the minimum image and the
         // pair uses the exact integer separation instead.
-        const bool wide = T(2) * (T)(E.x + E.y + E.z) + hT >= T(0.45) * (T)B.L;
-        T pw = 0, pdw = 0, pmw = 0, pmdw = 0;
+        const bool wide = 2.f * (E.x + E.y + E.z) + h >= 0.45f * B.Lf;
+        float pw = 0, pdw = 0, pmw = 0, pmdw = 0;
         for (long long q = q0; q < q1; ++q) {
-            T dx, dy, dz, m;
-            if (std::is_same<T, float>::value && !wide) {
+            float dx, dy, dz, m;
+            if (!wide) {
                 const float4 f = a.posf[q];
                 dx = ox + f.x; dy = oy + f.y; dz = oz + f.z; m = f.w;
             } else {
                 const uint4 Xj = a.posm[q];
-                dx = (T)(int)(Xj.x - Xi.x) * sT; dy = (T)(int)(Xj.y - Xi.y) * sT; dz = (T)(int)(Xj.z - Xi.z) * sT;
-                m = (T)__uint_as_float(Xj.w);
+                dx = (float)(int)(Xj.x - Xi.x) * sf; dy = (float)(int)(Xj.y - Xi.y) * sf; dz = (float)(int)(Xj.z - Xi.z) * sf;
+                m = __uint_as_float(Xj.w);
             }
-            const T r2 = dx * dx + dy * dy + dz * dz;
+            const float r2 = dx * dx + dy * dy + dz * dz;
             if (r2 < hi2) {
                 bool in = r2 < lo2;
                 if (!in) {
@@ -197,10 +145,10 @@ __device__ __forceinline__ void tpp_density_walk(const TppDensArgs& a, const Box
                     in = exact_pred(exact_d2(Xi, a.posm[q]), HH);
                 }
                 if (in) {
-                    const T qq = tpp_sqrt<T>(r2) * hinv;
-                    T w, dw;
-                    spline<T>(qq, w, dw);
-                    const T qdw = qq * dw;
+                    const float qq = tpp_sqrt(r2) * hinv;
+                    float w, dw;
+                    spline<float>(qq, w, dw);
+                    const float qdw = qq * dw;
                     pw += w;
                     pdw += qdw;
                     pmw += m * w;
@@ -236,7 +184,7 @@ __device__ float tpp_guess_h(const BoxDesc& B, const uint4* node_lo, const uint4
     return (float)best;
 }
 
-template <typename T, bool HASH>
+template <bool HASH>
 __global__ void __launch_bounds__(kTppThreads) k_density_tpp(TppDensArgs a) {
     const int cnt = a.count_ptr ? *a.count_ptr : a.count;
     unsigned long long c_pairs = 0, c_evals = 0, c_tests = 0;
@@ -253,13 +201,13 @@ __global__ void __launch_bounds__(kTppThreads) k_density_tpp(TppDensArgs a) {
         double blo = 0.0, bhi = INFINITY;
         float dold = INFINITY;
         unsigned st = 0;
-        TppDSums<T> S;
+        TppDSums S;
         for (int it = 0;; ++it) {
             S.sw = S.cw = S.sdw = S.cdw = S.smw = S.cmw = S.smdw = S.cmdw = 0;
             S.nn = 0;
             S.hs = 0;
             S.tests = 0;
-            tpp_density_walk<T, HASH>(a, B, p, Xi, h, S);
+            tpp_density_walk<HASH>(a, B, p, Xi, h, S);
             ++c_evals;
             c_tests += S.tests;
             const double f = (32.0 / 3.0) * ((double)S.sw - (double)S.cw) - a.n_target;
@@ -473,12 +421,12 @@ __global__ void __launch_bounds__(kTppThreads) k_density_buf(TppDensArgs a) {
         if (exact_finish) {
             // exact walk at the h reached, iterating further if needed
             for (;;) {
-                TppDSums<float> S;
+                TppDSums S;
                 S.sw = S.cw = S.sdw = S.cdw = S.smw = S.cmw = S.smdw = S.cmdw = 0.f;
                 S.nn = 0;
                 S.hs = 0;
                 S.tests = 0;
-                tpp_density_walk<float, HASH>(a, B, p, Xi, h, S);
+                tpp_density_walk<HASH>(a, B, p, Xi, h, S);
                 ++c_evals;
                 c_tests += S.tests;
                 smw = (double)S.smw - (double)S.cmw;
@@ -575,159 +523,6 @@ struct TppForceArgs {
     double alpha, gamma;
     Counters* ctr;
 };
-
-template <typename T, bool HASH>
-__global__ void __launch_bounds__(kTppThreads) k_force_tpp(TppForceArgs a) {
-    const int cnt = a.count_ptr ? *a.count_ptr : a.count;
-    const T alpha = (T)a.alpha, gam = (T)a.gamma, gm1 = (T)(a.gamma - 1.0);
-    const T kNorm = (T)(8.0 / 3.141592653589793);
-    unsigned long long c_pairs = 0, c_tests = 0;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x) {
-        const int p = a.act[t];
-        const BoxDesc& B = a.boxes[a.n_boxes == 1 ? 0 : tpp_box_of(a.boxes, a.n_boxes, p)];
-        const double L = B.L, s = ldexp(L, -32);
-        const float sf = (float)s;
-        const T sT = (T)s;
-        const uint4 Xi = a.posm[p];
-        const int oi = a.perm[p];
-        const float4 vi = a.fvel[p];
-        const float4 thi = a.fthermo[p];
-        const T hi = (T)vi.w, hinvi = T(1) / hi, rhoi = (T)thi.x;
-        T Ai, ci;
-        if constexpr (std::is_same<T, float>::value) {
-            Ai = thi.y;
-            ci = thi.z;
-        } else {
-            const T Pi = gm1 * rhoi * (T)a.u[oi];
-            Ai = (T)a.omega[oi] * Pi / (rhoi * rhoi);
-            ci = sqrt(gam * Pi / rhoi);
-        }
-        const T normi = kNorm * hinvi * hinvi * hinvi * hinvi;
-        const double Hd = (double)vi.w * 4294967296.0 / L;
-        const double HHi = Hd * Hd;
-        const T vxi = (T)vi.x, vyi = (T)vi.y, vzi = (T)vi.z;
-        T Sx = 0, Cx = 0, Sy = 0, Cy = 0, Sz = 0, Cz = 0, vsmax = 0;
-        double du = 0.0;
-        int np = 0;
-        unsigned long long hs = 0, tests = 0;
-
-        int stack[kTppStack];
-        int sp = 0;
-        stack[sp++] = B.nlev == 1 ? 0 : (B.nlev - 1) << 27;
-        const long long pend = B.off + B.n;
-        while (sp > 0) {
-            const int enc = stack[--sp];
-            const int lev = enc >> 27, tt = enc & ((1 << 27) - 1);
-            if (lev > 0) {
-                const int cl = lev - 1;
-                const int c0 = tt * kFan, c1 = min(c0 + kFan, B.lvl_n[cl]);
-                const int base = B.lvl_off[cl];
-                for (int c = c0; c < c1; ++c) {
-                    const float4 e = a.node_e[base + c];
-                    if (tpp_node_near(a.node_c[base + c], e, Xi, sf, fmaxf(vi.w, e.w))) stack[sp++] = (cl << 27) | c;
-                }
-                continue;
-            }
-            const int nd = B.lvl_off[0] + tt;
-            const uint4 C = a.node_c[nd];
-            const float4 E = a.node_e[nd];
-            const T ox = (T)(int)(C.x - Xi.x) * sT, oy = (T)(int)(C.y - Xi.y) * sT, oz = (T)(int)(C.z - Xi.z) * sT;
-            const T eL = TBand<T>::rel * (T(4) * (T)(E.x + E.y + E.z) + T(2) * (fabs(ox) + fabs(oy) + fabs(oz)));
-            const T elo = T(1) - T(4) * TBand<T>::rel, ehi = T(1) + T(4) * TBand<T>::rel;
-            const T ei = eL + TBand<T>::rel * T(2) * hi;
-            const T lo2i = hi > ei ? (hi - ei) * (hi - ei) * elo : T(0);
-            const T hi2i = (hi + ei) * (hi + ei) * ehi;
-            const long long q0 = B.off + (long long)tt * kLeaf, q1 = min(q0 + kLeaf, pend);
-            // leaves wider than the minimum-image sum allows: exact integer separations
-            const bool wide = T(2) * (T)(E.x + E.y + E.z) + max(hi, (T)E.w) >= T(0.45) * (T)B.L;
-            T pax = 0, pay = 0, paz = 0, pdu = 0;
-            for (long long q = q0; q < q1; ++q) {
-                if (q == p) continue;
-                T dx, dy, dz, mj;   // d = x_j - x_i
-                if (std::is_same<T, float>::value && !wide) {
-                    const float4 f = a.posf[q];
-                    dx = ox + f.x; dy = oy + f.y; dz = oz + f.z; mj = f.w;
-                } else {
-                    const uint4 Xj = a.posm[q];
-                    dx = (T)(int)(Xj.x - Xi.x) * sT; dy = (T)(int)(Xj.y - Xi.y) * sT; dz = (T)(int)(Xj.z - Xi.z) * sT;
-                    mj = (T)__uint_as_float(Xj.w);
-                }
-                const T r2 = dx * dx + dy * dy + dz * dz;
-                const float4 vj = a.fvel[q];
-                const T hj = (T)vj.w;
-                const T ej = eL + TBand<T>::rel * T(2) * hj;
-                const T hi2j = (hj + ej) * (hj + ej) * ehi;
-                const bool mi = r2 < hi2i, mjb = r2 < hi2j;
-                if (!(mi || mjb)) continue;
-                bool in = r2 < lo2i || r2 < (hj > ej ? (hj - ej) * (hj - ej) * elo : T(0));
-                if (!in) {
-                    const unsigned long long D2 = exact_d2(Xi, a.posm[q]);
-                    const double Hj = (double)vj.w * 4294967296.0 / L;
-                    in = (mi && exact_pred(D2, HHi)) || (mjb && exact_pred(D2, Hj * Hj));
-                }
-                if (!in) continue;
-                ++np;
-                if (HASH) hs += splitmix64((unsigned long long)a.perm[q]);
-                const float4 thj = a.fthermo[q];
-                T Aj, cj, hinvj;
-                const T rhoj = (T)thj.x;
-                if constexpr (std::is_same<T, float>::value) {
-                    Aj = thj.y; cj = thj.z; hinvj = thj.w;
-                } else {
-                    const int o = a.perm[q];
-                    const T Pj = gm1 * rhoj * (T)a.u[o];
-                    Aj = (T)a.omega[o] * Pj / (rhoj * rhoj);
-                    cj = sqrt(gam * Pj / rhoj);
-                    hinvj = T(1) / hj;
-                }
-                if (r2 <= T(0)) {  // coincident: no direction, no force
-                    vsmax = max(vsmax, ci + cj);
-                    continue;
-                }
-                T rinv;
-                if constexpr (std::is_same<T, float>::value) rinv = rsqrtf(r2);
-                else rinv = 1.0 / sqrt(r2);
-                const T r = r2 * rinv;
-                T w_, dwi, dwj;
-                spline<T>(r * hinvi, w_, dwi);
-                spline<T>(r * hinvj, w_, dwj);
-                const T Fi = normi * dwi * rinv;
-                const T Fj = kNorm * hinvj * hinvj * hinvj * hinvj * dwj * rinv;
-                // r_ij = x_i - x_j = -d ; v_ij = v_i - v_j
-                const T vr = -((vxi - (T)vj.x) * dx + (vyi - (T)vj.y) * dy + (vzi - (T)vj.z) * dz);
-                const T wij = vr * rinv;
-                const T vs = ci + cj - T(3) * wij;
-                vsmax = max(vsmax, vs);
-                const T PI = wij < T(0) ? -alpha * vs * wij / (rhoi + rhoj) : T(0);
-                const T Fbar = T(0.5) * (Fi + Fj);
-                const T coef = mj * (Ai * Fi + Aj * Fj + PI * Fbar);
-                pax += coef * dx;   // -coef * r_ij
-                pay += coef * dy;
-                paz += coef * dz;
-                pdu += mj * vr * (Ai * Fi + T(0.5) * PI * Fbar);
-            }
-            tests += (unsigned long long)(q1 - q0);
-            kahan_add(Sx, Cx, pax);
-            kahan_add(Sy, Cy, pay);
-            kahan_add(Sz, Cz, paz);
-            du += (double)pdu;
-        }
-        a.acc[3 * (size_t)oi] = (float)((double)Sx - (double)Cx);
-        a.acc[3 * (size_t)oi + 1] = (float)((double)Sy - (double)Cy);
-        a.acc[3 * (size_t)oi + 2] = (float)((double)Sz - (double)Cz);
-        a.dudt[oi] = (float)du;
-        a.vsig[oi] = (float)vsmax;
-        if (HASH) a.hash[oi] = hs;
-        c_pairs += (unsigned long long)np;
-        c_tests += tests;
-    }
-    c_pairs = warp_sum(c_pairs);
-    c_tests = warp_sum(c_tests);
-    if (lane_id() == 0) {
-        atomicAdd(&a.ctr->force_pairs, c_pairs);
-        atomicAdd(&a.ctr->pair_tests, c_tests);
-    }
-}
 
 // FP32 force (default): while-while walk; per leaf a cheap membership pass
 // builds a bit mask of the pairs in the symmetric set, then the expensive
@@ -918,12 +713,9 @@ cudaError_t launch_density_tpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
     da.guess_h = a.guess_h;
     da.ctr = ctx->counters;
     const int blocks = tpp_blocks(ctx, a.blocks_per_sm, n_active);
-    if (a.fp64)
-        return a.hash ? timed_launch(ctx, k_density_tpp<double, true>, da, blocks, 0, a.time_kernels, s)
-                      : timed_launch(ctx, k_density_tpp<double, false>, da, blocks, 0, a.time_kernels, s);
     if (a.hash || a.fixed_h || !a.buffered)
-        return a.hash ? timed_launch(ctx, k_density_tpp<float, true>, da, blocks, 0, a.time_kernels, s)
-                      : timed_launch(ctx, k_density_tpp<float, false>, da, blocks, 0, a.time_kernels, s);
+        return a.hash ? timed_launch(ctx, k_density_tpp<true>, da, blocks, 0, a.time_kernels, s)
+                      : timed_launch(ctx, k_density_tpp<false>, da, blocks, 0, a.time_kernels, s);
     return timed_launch(ctx, k_density_buf<false>, da, blocks, 0, a.time_kernels, s);
 }
 
@@ -965,9 +757,6 @@ cudaError_t launch_force_tpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_activ
     fa.gamma = a.gamma;
     fa.ctr = ctx->counters;
     const int blocks = tpp_blocks(ctx, a.blocks_per_sm, n_active);
-    if (a.fp64)
-        return a.hash ? timed_launch(ctx, k_force_tpp<double, true>, fa, blocks, 1, a.time_kernels, s)
-                      : timed_launch(ctx, k_force_tpp<double, false>, fa, blocks, 1, a.time_kernels, s);
     return a.hash ? timed_launch(ctx, k_force_mask<true>, fa, blocks, 1, a.time_kernels, s)
                   : timed_launch(ctx, k_force_mask<false>, fa, blocks, 1, a.time_kernels, s);
 }
