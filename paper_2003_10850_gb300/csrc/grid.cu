@@ -444,83 +444,138 @@ __device__ __forceinline__ void node_geom(uint4 a, uint4 b, double s, uint4& c, 
                     (float)((double)(((b.z - a.z) >> 1) + 2u) * s), 0.f);
 }
 
-__global__ void k_leaf_bbox(const uint4* __restrict__ posm, const BoxDesc* __restrict__ boxes,
-                            uint4* __restrict__ lo, uint4* __restrict__ hi, uint4* __restrict__ nc,
-                            float4* __restrict__ ne, float4* __restrict__ posf) {
-    const BoxDesc& B = boxes[blockIdx.y];
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.lvl_n[0]) return;
-    long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
-    uint4 a = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0), b = make_uint4(0, 0, 0, 0);
-    for (long long p = p0; p < p1; ++p) {
-        uint4 x = posm[p];
-        a.x = min(a.x, x.x); a.y = min(a.y, x.y); a.z = min(a.z, x.z);
-        b.x = max(b.x, x.x); b.y = max(b.y, x.y); b.z = max(b.z, x.z);
-    }
-    const int nd = B.lvl_off[0] + t;
-    lo[nd] = a;
-    hi[nd] = b;
-    const double s = ldexp(B.L, -32);
-    uint4 c;
+// The hierarchy is built in two launches: blocks of kTreeT leaves form levels
+// 0 to 2 of their part (a level's results pass through shared memory), then one
+// block per box forms the few nodes of the levels above, one level after another.
+// (One launch per level, most of them a handful of threads, took five to seven.)
+
+// Bounds and geometry of node nd.
+__device__ __forceinline__ void put_bbox(int nd, uint4 a, uint4 b, double s, uint4* __restrict__ lo,
+                                         uint4* __restrict__ hi, uint4* __restrict__ nc, float4* __restrict__ ne,
+                                         uint4& c) {
     float4 e;
     node_geom(a, b, s, c, e);
-    nc[nd] = c;
-    ne[nd] = e;
-    // leaf-relative FP32 coordinates (box units) and mass of the leaf's particles
-    const float sf = (float)s;
-    for (long long p = p0; p < p1; ++p) {
-        uint4 x = posm[p];
-        posf[p] = make_float4((float)(int)(x.x - c.x) * sf, (float)(int)(x.y - c.y) * sf,
-                              (float)(int)(x.z - c.z) * sf, __uint_as_float(x.w));
-    }
-}
-
-__global__ void k_node_bbox(int lev, const BoxDesc* __restrict__ boxes, uint4* __restrict__ lo,
-                            uint4* __restrict__ hi, uint4* __restrict__ nc, float4* __restrict__ ne) {
-    const BoxDesc& B = boxes[blockIdx.y];
-    if (lev >= B.nlev) return;
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.lvl_n[lev]) return;
-    int c0 = t * kFan, c1 = min(c0 + kFan, B.lvl_n[lev - 1]);
-    uint4 a = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0), b = make_uint4(0, 0, 0, 0);
-    for (int c = c0; c < c1; ++c) {
-        uint4 x = lo[B.lvl_off[lev - 1] + c], y = hi[B.lvl_off[lev - 1] + c];
-        a.x = min(a.x, x.x); a.y = min(a.y, x.y); a.z = min(a.z, x.z);
-        b.x = max(b.x, y.x); b.y = max(b.y, y.y); b.z = max(b.z, y.z);
-    }
-    const int nd = B.lvl_off[lev] + t;
     lo[nd] = a;
     hi[nd] = b;
-    uint4 c;
-    float4 e;
-    node_geom(a, b, ldexp(B.L, -32), c, e);
     nc[nd] = c;
     ne[nd] = e;
 }
-
-__global__ void k_leaf_hmax(const int32_t* __restrict__ perm, const float* __restrict__ h,
-                            const BoxDesc* __restrict__ boxes, float* __restrict__ hmax, float4* __restrict__ ne) {
-    const BoxDesc& B = boxes[blockIdx.y];
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.lvl_n[0]) return;
-    long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
-    float m = 0.f;
-    for (long long p = p0; p < p1; ++p) m = fmaxf(m, h[perm[p]]);
-    hmax[B.lvl_off[0] + t] = m;
-    ne[B.lvl_off[0] + t].w = m;
+__device__ __forceinline__ void join_bbox(uint4& a, uint4& b, uint4 x, uint4 y) {
+    a.x = min(a.x, x.x); a.y = min(a.y, x.y); a.z = min(a.z, x.z);
+    b.x = max(b.x, y.x); b.y = max(b.y, y.y); b.z = max(b.z, y.z);
 }
 
-__global__ void k_node_hmax(int lev, const BoxDesc* __restrict__ boxes, float* __restrict__ hmax,
-                            float4* __restrict__ ne) {
+__global__ void __launch_bounds__(kTreeT) k_tree_low(const uint4* __restrict__ posm, const BoxDesc* __restrict__ boxes,
+                                                     uint4* __restrict__ lo, uint4* __restrict__ hi,
+                                                     uint4* __restrict__ nc, float4* __restrict__ ne,
+                                                     float4* __restrict__ posf) {
+    __shared__ uint4 sa[kTreeT], sb[kTreeT];
     const BoxDesc& B = boxes[blockIdx.y];
-    if (lev >= B.nlev) return;
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.lvl_n[lev]) return;
-    int c0 = t * kFan, c1 = min(c0 + kFan, B.lvl_n[lev - 1]);
+    const int tid = threadIdx.x, t = blockIdx.x * kTreeT + tid;
+    if (blockIdx.x * kTreeT >= B.lvl_n[0]) return;
+    const double s = ldexp(B.L, -32);
+    const uint4 a0 = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0), b0 = make_uint4(0, 0, 0, 0);
+    uint4 a = a0, b = b0, c;
+    if (t < B.lvl_n[0]) {
+        const long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
+        for (long long p = p0; p < p1; ++p) {
+            const uint4 x = posm[p];
+            join_bbox(a, b, x, x);
+        }
+        put_bbox(B.lvl_off[0] + t, a, b, s, lo, hi, nc, ne, c);
+        // leaf-relative FP32 coordinates (box units) and mass of the leaf's particles
+        const float sf = (float)s;
+        for (long long p = p0; p < p1; ++p) {
+            const uint4 x = posm[p];
+            posf[p] = make_float4((float)(int)(x.x - c.x) * sf, (float)(int)(x.y - c.y) * sf,
+                                  (float)(int)(x.z - c.z) * sf, __uint_as_float(x.w));
+        }
+    }
+    sa[tid] = a;
+    sb[tid] = b;
+    int w = kTreeT;
+#pragma unroll
+    for (int lev = 1; lev < kTreeLow; ++lev) {
+        w /= kFan;
+        __syncthreads();
+        const int tt = blockIdx.x * w + tid;
+        a = a0;
+        b = b0;
+        if (tid < w)   // (children past the level's end hold the neutral bounds)
+            for (int k = 0; k < kFan; ++k) join_bbox(a, b, sa[tid * kFan + k], sb[tid * kFan + k]);
+        __syncthreads();
+        if (tid < w) {
+            sa[tid] = a;
+            sb[tid] = b;
+            if (lev < B.nlev && tt < B.lvl_n[lev]) put_bbox(B.lvl_off[lev] + tt, a, b, s, lo, hi, nc, ne, c);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kTreeTopT) k_tree_top(const BoxDesc* __restrict__ boxes, uint4* lo, uint4* hi,
+                                                        uint4* __restrict__ nc, float4* __restrict__ ne) {
+    const BoxDesc& B = boxes[blockIdx.x];
+    const double s = ldexp(B.L, -32);
+    for (int lev = kTreeLow; lev < B.nlev; ++lev) {
+        for (int t = threadIdx.x; t < B.lvl_n[lev]; t += kTreeTopT) {
+            const int c0 = t * kFan, c1 = min(c0 + kFan, B.lvl_n[lev - 1]);
+            uint4 a = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0), b = make_uint4(0, 0, 0, 0), c;
+            for (int k = c0; k < c1; ++k) join_bbox(a, b, lo[B.lvl_off[lev - 1] + k], hi[B.lvl_off[lev - 1] + k]);
+            put_bbox(B.lvl_off[lev] + t, a, b, s, lo, hi, nc, ne, c);
+        }
+        __syncthreads();
+    }
+}
+
+// h_max of every node, as the bounds.
+__global__ void __launch_bounds__(kTreeT) k_hmax_low(const int32_t* __restrict__ perm, const float* __restrict__ h,
+                                                     const BoxDesc* __restrict__ boxes, float* __restrict__ hmax,
+                                                     float4* __restrict__ ne) {
+    __shared__ float sm[kTreeT];
+    const BoxDesc& B = boxes[blockIdx.y];
+    const int tid = threadIdx.x, t = blockIdx.x * kTreeT + tid;
+    if (blockIdx.x * kTreeT >= B.lvl_n[0]) return;
     float m = 0.f;
-    for (int c = c0; c < c1; ++c) m = fmaxf(m, hmax[B.lvl_off[lev - 1] + c]);
-    hmax[B.lvl_off[lev] + t] = m;
-    ne[B.lvl_off[lev] + t].w = m;
+    if (t < B.lvl_n[0]) {
+        const long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
+        for (long long p = p0; p < p1; ++p) m = fmaxf(m, h[perm[p]]);
+        hmax[B.lvl_off[0] + t] = m;
+        ne[B.lvl_off[0] + t].w = m;
+    }
+    sm[tid] = m;
+    int w = kTreeT;
+#pragma unroll
+    for (int lev = 1; lev < kTreeLow; ++lev) {
+        w /= kFan;
+        __syncthreads();
+        const int tt = blockIdx.x * w + tid;
+        m = 0.f;
+        if (tid < w)
+            for (int k = 0; k < kFan; ++k) m = fmaxf(m, sm[tid * kFan + k]);
+        __syncthreads();
+        if (tid < w) {
+            sm[tid] = m;
+            if (lev < B.nlev && tt < B.lvl_n[lev]) {
+                hmax[B.lvl_off[lev] + tt] = m;
+                ne[B.lvl_off[lev] + tt].w = m;
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kTreeTopT) k_hmax_top(const BoxDesc* __restrict__ boxes, float* hmax,
+                                                        float4* __restrict__ ne) {
+    const BoxDesc& B = boxes[blockIdx.x];
+    for (int lev = kTreeLow; lev < B.nlev; ++lev) {
+        for (int t = threadIdx.x; t < B.lvl_n[lev]; t += kTreeTopT) {
+            const int c0 = t * kFan, c1 = min(c0 + kFan, B.lvl_n[lev - 1]);
+            float m = 0.f;
+            for (int c = c0; c < c1; ++c) m = fmaxf(m, hmax[B.lvl_off[lev - 1] + c]);
+            hmax[B.lvl_off[lev] + t] = m;
+            ne[B.lvl_off[lev] + t].w = m;
+        }
+        __syncthreads();
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -594,12 +649,11 @@ static cudaError_t grid_fill(sph_grid* g, const void* pos, int f64, const float*
                                   ctx->counters, s, &ctx->launches);
     if (e) return e;
     k_gather<<<blocks, 256, 0, s>>>(g->xq, n, g->posm, g->perm, g->rank);
-    dim3 lg((g->max_leaves + 127) / 128, nb);
-    k_leaf_bbox<<<lg, 128, 0, s>>>(g->posm, g->boxes, g->node_lo, g->node_hi, g->node_c, g->node_e, g->posf);
+    k_tree_low<<<dim3((g->max_leaves + kTreeT - 1) / kTreeT, nb), kTreeT, 0, s>>>(
+        g->posm, g->boxes, g->node_lo, g->node_hi, g->node_c, g->node_e, g->posf);
     ctx->launches += 2;
-    for (int lev = 1; lev < g->max_lev; ++lev) {
-        dim3 ng((g->lvl_max[lev] + 127) / 128, nb);
-        k_node_bbox<<<ng, 128, 0, s>>>(lev, g->boxes, g->node_lo, g->node_hi, g->node_c, g->node_e);
+    if (g->max_lev > kTreeLow) {
+        k_tree_top<<<nb, kTreeTopT, 0, s>>>(g->boxes, g->node_lo, g->node_hi, g->node_c, g->node_e);
         ++ctx->launches;
     }
     return cudaGetLastError();
@@ -745,12 +799,11 @@ sph_status grid_update(sph_grid* g, const void* pos, int f64, const float* mass,
 
 void grid_refresh_hmax(sph_grid* g, const float* h, cudaStream_t s) {
     int nb = g->n_boxes;
-    dim3 lg((g->max_leaves + 127) / 128, nb);
-    k_leaf_hmax<<<lg, 128, 0, s>>>(g->perm, h, g->boxes, g->node_hmax, g->node_e);
+    k_hmax_low<<<dim3((g->max_leaves + kTreeT - 1) / kTreeT, nb), kTreeT, 0, s>>>(g->perm, h, g->boxes, g->node_hmax,
+                                                                              g->node_e);
     ++g->ctx->launches;
-    for (int lev = 1; lev < g->max_lev; ++lev) {
-        dim3 ng((g->lvl_max[lev] + 127) / 128, nb);
-        k_node_hmax<<<ng, 128, 0, s>>>(lev, g->boxes, g->node_hmax, g->node_e);
+    if (g->max_lev > kTreeLow) {
+        k_hmax_top<<<nb, kTreeTopT, 0, s>>>(g->boxes, g->node_hmax, g->node_e);
         ++g->ctx->launches;
     }
 }

@@ -126,6 +126,9 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
                       const int64_t* offs, const double* Ls, int nb, cudaStream_t s,
                       sph_grid** out);
 void grid_free(sph_grid* g);
+// hierarchy passes: leaves per block of the first kernel, levels it forms, threads per box of the second
+constexpr int kTreeT = 256, kTreeLow = 3, kTreeTopT = 512;
+static_assert(kTreeT % (kFan * kFan) == 0, "whole level-2 nodes per block");
 // re-quantise, re-sort and rebuild the hierarchy in place (same n and boxes)
 sph_status grid_update(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s);
 // hmax of every node from the caller-order h
