@@ -20,12 +20,17 @@
 // each if its coarse distance is below RCi). D2 < RCi <= 2^44 and P <= 2^16
 // keep the products below 2^60.
 //
-// One warp per active particle: each step pops up to four opened nodes and
-// tests their children one per lane; opened leaves gather in a shared list
-// whose particles are tested four leaves at a time (lanes 8k..8k+7 on leaf
-// k). Accepted nodes and particles inside the cutoff are compacted by ballot
-// into a per-warp interaction buffer that is evaluated 32 entries at a time,
-// so the pair terms run with every lane busy. The pair term is
+// A warp walks for a group of up to M active particles (its members) of one
+// aligned run of 64 sorted particles, 32/M lanes serving each member:
+// - a step pops up to four opened nodes and tests their children, one per lane,
+//   against every member, in FP32 where that settles the exact rule and by the
+//   rule itself elsewhere (see grav_decide); a child that some member opens is
+//   pushed with its member mask, and a member that accepts a node or opens a leaf
+//   puts it on its own list;
+// - a full list is worked off by the lanes of its member: accepted nodes, and the
+//   particles of opened leaves, each inside the cutoff by an FP32 test of the
+//   separation that the pair term needs anyway (the exact test in a thin band).
+// The pair term is
 //   a_i += G m_j K(r) (x_j - x_i),  K(r) = M(r/h_s) g(r) / r^3,
 // M the spline softening's mass fraction, g(r) = erfc(r/2r_s) + r/(r_s sqrt(pi))
 // exp(-r^2/4r_s^2) the short-range factor (erfc to 1.5e-7, see grav_K).
@@ -36,13 +41,21 @@
 namespace sph {
 
 constexpr int kGravStack = 256;   // see the bound below
-constexpr int kGravLeaves = 64;   // opened leaves waiting; <= 3 + 32 at any time
-constexpr int kGravHits = 64;     // interactions waiting; <= 31 + 32 at any time
+constexpr int kGravLeaves = 128;  // opened leaves waiting per member; a step adds <= 32
+constexpr int kGravNodes = 64;    // accepted nodes waiting per member; a step adds <= 32
 
 // Stack bound: a pop-4 step starts at sp <= 96 and pushes <= 32 children; in
 // the pop-1 regime a step pushes <= 8 children of the node it pops, so the
 // stack grows by at most 7 per level of depth-first descent:
 // sp <= 124 + 7 kMaxLev < kGravStack.
+
+struct GravBox {
+    unsigned long long RCi;
+    float rcu;               // 256 sqrt(RCi): the cutoff in integer units
+    float r2_in, r2_out;     // squared separation (box units): surely inside below, surely outside above
+    float pad;
+};
+static_assert(sizeof(GravBox) == kGravBoxBytes, "the grid's per-box gravity store");
 
 struct GravArgs {
     const BoxDesc* boxes;
@@ -56,97 +69,164 @@ struct GravArgs {
     const uint4* node_hi;
     const uint4* node_c;
     const float4* node_m;   // centre of mass - node centre (box units), mass
-    const unsigned long long* box_rci;   // per box: RCi
+    const GravBox* gbox;    // per box: the cutoff
     float* acc;
     int32_t* n_nodes;
     int32_t* n_pairs;
     Counters* ctr;
     float G;
     unsigned long long P;    // rint(theta^2 2^16)
+    float inv_theta;         // 256 / sqrt(P) (P = 0: unused)
     float hs, inv_hs;        // softening radius (0: none)
     float inv2rs;            // 1 / (2 r_s); r_s <= 0: 0
 };
 
-// Leaf moments: mass and centre of mass relative to the node centre.
-__global__ void k_grav_leaf_moments(const uint4* __restrict__ posm, const BoxDesc* __restrict__ boxes,
-                                    const uint4* __restrict__ nc, float4* __restrict__ nm) {
-    const BoxDesc& B = boxes[blockIdx.y];
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.lvl_n[0]) return;
-    const long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
-    const int nd = B.lvl_off[0] + t;
-    const uint4 c = nc[nd];
-    float M = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
-    for (long long p = p0; p < p1; ++p) {
-        const uint4 x = posm[p];
-        const float m = __uint_as_float(x.w);
-        M += m;
-        sx = fmaf(m, (float)(int)(x.x - c.x), sx);
-        sy = fmaf(m, (float)(int)(x.y - c.y), sy);
-        sz = fmaf(m, (float)(int)(x.z - c.z), sz);
-    }
-    const float s = M > 0.f ? B.sf / M : 0.f;
-    nm[nd] = make_float4(sx * s, sy * s, sz * s, M);
-}
-
-// Node moments from the children's (level lev >= 1).
-__global__ void k_grav_node_moments(int lev, const BoxDesc* __restrict__ boxes, const uint4* __restrict__ nc,
-                                    float4* __restrict__ nm) {
-    const BoxDesc& B = boxes[blockIdx.y];
-    if (lev >= B.nlev) return;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B.lvl_n[lev]) return;
-    const int c0 = t * kFan, c1 = min(c0 + kFan, B.lvl_n[lev - 1]);
-    const int nd = B.lvl_off[lev] + t;
-    const uint4 c = nc[nd];
-    const float sf = B.sf;
+// Mass and centre of mass relative to the node centre of a node whose children
+// c0..c1 are in (q: moments, cc: centres), in order.
+template <class Q, class C>
+__device__ __forceinline__ float4 grav_join(int c0, int c1, uint4 c, float sf, Q&& q_, C&& cc_) {
     float M = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
     for (int k = c0; k < c1; ++k) {
-        const int ch = B.lvl_off[lev - 1] + k;
-        const float4 q = nm[ch];
-        const uint4 cc = nc[ch];
+        const float4 q = q_(k);
+        const uint4 cc = cc_(k);
         M += q.w;
         sx = fmaf(q.w, fmaf((float)(int)(cc.x - c.x), sf, q.x), sx);
         sy = fmaf(q.w, fmaf((float)(int)(cc.y - c.y), sf, q.y), sy);
         sz = fmaf(q.w, fmaf((float)(int)(cc.z - c.z), sf, q.z), sz);
     }
     const float s = M > 0.f ? 1.f / M : 0.f;
-    nm[nd] = make_float4(sx * s, sy * s, sz * s, M);
+    return make_float4(sx * s, sy * s, sz * s, M);
 }
 
-// RCi = ceil((r_cut 2^24 / L)^2) of each box (FP64, then exact).
-__global__ void k_grav_box_rc(const BoxDesc* __restrict__ boxes, int nb, double r_cut,
-                              unsigned long long* __restrict__ rci) {
+// Moments of levels 0 to 2, a block per kTreeT leaves (as the bounds, see grid.cu).
+__global__ void __launch_bounds__(kTreeT) k_grav_low(const uint4* __restrict__ posm, const BoxDesc* __restrict__ boxes,
+                                                     const uint4* __restrict__ nc, float4* __restrict__ nm) {
+    __shared__ float4 sq[kTreeT];
+    __shared__ uint4 sc[kTreeT];
+    const BoxDesc& B = boxes[blockIdx.y];
+    const int tid = threadIdx.x, t = blockIdx.x * kTreeT + tid;
+    if (blockIdx.x * kTreeT >= B.lvl_n[0]) return;
+    const float sf = B.sf;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint4 c = make_uint4(0u, 0u, 0u, 0u);
+    if (t < B.lvl_n[0]) {
+        const long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
+        const int nd = B.lvl_off[0] + t;
+        c = nc[nd];
+        float M = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
+        for (long long p = p0; p < p1; ++p) {
+            const uint4 x = posm[p];
+            const float m = __uint_as_float(x.w);
+            M += m;
+            sx = fmaf(m, (float)(int)(x.x - c.x), sx);
+            sy = fmaf(m, (float)(int)(x.y - c.y), sy);
+            sz = fmaf(m, (float)(int)(x.z - c.z), sz);
+        }
+        const float s = M > 0.f ? sf / M : 0.f;
+        q = make_float4(sx * s, sy * s, sz * s, M);
+        nm[nd] = q;
+    }
+    sq[tid] = q;
+    sc[tid] = c;
+    int w = kTreeT;
+#pragma unroll
+    for (int lev = 1; lev < kTreeLow; ++lev) {
+        w /= kFan;
+        __syncthreads();
+        const int tt = blockIdx.x * w + tid;
+        const bool live = tid < w && lev < B.nlev && tt < B.lvl_n[lev];
+        if (live) {
+            const int c0 = tid * kFan, c1 = c0 + min(kFan, B.lvl_n[lev - 1] - tt * kFan);
+            c = nc[B.lvl_off[lev] + tt];
+            q = grav_join(c0, c1, c, sf, [&](int k) { return sq[k]; }, [&](int k) { return sc[k]; });
+            nm[B.lvl_off[lev] + tt] = q;
+        }
+        __syncthreads();
+        if (live) {
+            sq[tid] = q;
+            sc[tid] = c;
+        }
+    }
+}
+
+// The levels above, a block per box.
+__global__ void __launch_bounds__(kTreeTopT) k_grav_top(const BoxDesc* __restrict__ boxes,
+                                                        const uint4* __restrict__ nc, float4* nm) {
+    const BoxDesc& B = boxes[blockIdx.x];
+    for (int lev = kTreeLow; lev < B.nlev; ++lev) {
+        const int below = B.lvl_off[lev - 1];
+        for (int t = threadIdx.x; t < B.lvl_n[lev]; t += kTreeTopT) {
+            const int nd = B.lvl_off[lev] + t;
+            nm[nd] = grav_join(t * kFan, min(t * kFan + kFan, B.lvl_n[lev - 1]), nc[nd], B.sf,
+                               [&](int k) { return nm[below + k]; }, [&](int k) { return nc[below + k]; });
+        }
+        __syncthreads();
+    }
+}
+
+// The cutoff of each box: RCi = ceil((r_cut 2^24 / L)^2) (FP64, then exact), its
+// radius in integer units, and the FP32 bounds of the particle test on the
+// squared separation in box units. A coarse distance is between the true one
+// less 256 sqrt(3) units and the true one, so below 256 sqrt(RCi) a particle is
+// inside and 444 units beyond it is outside; 2^-19 covers the FP32 rounding of
+// the squared separation. Box sizes whose squares leave the FP32 range take the
+// exact test always.
+__global__ void k_grav_box_rc(const BoxDesc* __restrict__ boxes, int nb, double r_cut, GravBox* __restrict__ gb) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
     const double rcu = r_cut / boxes[b].L * 16777216.0;
-    rci[b] = (unsigned long long)ceil(rcu * rcu);
+    GravBox g;
+    g.RCi = (unsigned long long)ceil(rcu * rcu);
+    const double rc = 256.0 * sqrt((double)g.RCi), s = boxes[b].L * 2.3283064365386962890625e-10;
+    const double lo = rc * s * rc * s * (1.0 - 1.9073486328125e-06), hi = (rc + 448.0) * s * (rc + 448.0) * s *
+                                                                         (1.0 + 1.9073486328125e-06);
+    const bool ok = lo > 1e-30 && hi < 1e30;
+    g.rcu = (float)rc;
+    g.r2_in = ok ? (float)lo : -1.f;
+    g.r2_out = ok ? (float)hi : INFINITY;
+    g.pad = 0.f;
+    gb[b] = g;
 }
 
-// M(q) g(r) / r^3 for r^2 = r2 > 0, and r.
+// Approximations without the denormal cases (none occur: r^3 stays far inside
+// the normal range and an exponential that small adds nothing).
+__device__ __forceinline__ float grav_ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Mass fraction of the cubic spline (support 1) inside q < 1.
+__device__ __forceinline__ float grav_soft(float q) {
+    const float q2 = q * q, q3 = q2 * q;
+    return q <= 0.5f ? q3 * fmaf(q2, fmaf(32.f, q, -192.f / 5.f), 32.f / 3.f)
+                     : fmaf(q3, fmaf(q, fmaf(q, fmaf(-32.f / 3.f, q, 192.f / 5.f), -48.f), 64.f / 3.f), -1.f / 15.f);
+}
+
+// M(q) g(r) / r^3 of two pairs, r^2 = r2 > 0.
 // The split factor g = erfc(x) + (2/sqrt(pi)) x e^{-x^2}, x = r / (2 r_s), takes
 // erfc from Abramowitz & Stegun 7.1.26 (Hastings' rational approximation,
 // |error| <= 1.5e-7): erfc(x) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) e^{-x^2},
 // t = 1 / (1 + p x), so that both terms share one exponential.
-__device__ __forceinline__ float grav_K(const GravArgs& a, float r2, float& r) {
-    r = r2 * rsqrtf(r2);
-    float Mq = 1.f;
-    if (r < a.hs) {   // mass fraction of the cubic spline (support 1) inside q
-        const float q = r * a.inv_hs, q2 = q * q, q3 = q2 * q;
-        Mq = q <= 0.5f ? q3 * fmaf(q2, fmaf(32.f, q, -192.f / 5.f), 32.f / 3.f)
-                       : fmaf(q3, fmaf(q, fmaf(q, fmaf(-32.f / 3.f, q, 192.f / 5.f), -48.f), 64.f / 3.f),
-                              -1.f / 15.f);
-    }
-    float g = 1.f;
+__device__ __forceinline__ float2 grav_K(const GravArgs& a, float2 r2) {
+    const float2 r = mul2(r2, make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)));
+    float2 K = both(1.f);
+    if (r.x < a.hs) K.x = grav_soft(r.x * a.inv_hs);
+    if (r.y < a.hs) K.y = grav_soft(r.y * a.inv_hs);
     if (a.inv2rs > 0.f) {
-        const float x = r * a.inv2rs;
-        const float t = __fdividef(1.f, fmaf(0.3275911f, x, 1.f));
-        const float poly =
-            t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f),
-                     0.254829592f);
-        g = __expf(-x * x) * fmaf(1.1283791671f, x, poly);   // 2 / sqrt(pi) = 1.1283791671
+        const float2 x = mul2(r, both(a.inv2rs));
+        const float2 y = fma2(both(0.3275911f), x, both(1.f));
+        const float2 t = make_float2(rcp_ftz(y.x), rcp_ftz(y.y));
+        float2 e = fma2(t, both(1.061405429f), both(-1.453152027f));
+        e = fma2(t, e, both(1.421413741f));
+        e = fma2(t, e, both(-0.284496736f));
+        e = fma2(t, e, both(0.254829592f));
+        e = fma2(both(1.1283791671f), x, mul2(t, e));   // 2 / sqrt(pi)
+        const float2 z = mul2(mul2(x, x), both(-1.4426950409f));   // log2 e
+        K = mul2(K, mul2(make_float2(grav_ex2(z.x), grav_ex2(z.y)), e));
     }
-    return __fdividef(Mq * g, r2 * r);   // r^3 stays far inside the normal range
+    const float2 r3 = mul2(r2, r);
+    return mul2(K, make_float2(rcp_ftz(r3.x), rcp_ftz(r3.y)));
 }
 
 // One axis of the exact coarse box geometry: squared gap, squared far-side
@@ -179,553 +259,298 @@ __device__ __forceinline__ void grav_box(uint4 X, uint4 lo, uint4 hi, unsigned l
     L2 = (unsigned long long)l * l;
 }
 
-__global__ void __launch_bounds__(kWppThreads) k_gravity(GravArgs a) {
-    __shared__ int stk_all[kWppWarps][kGravStack];
-    __shared__ int lf_all[kWppWarps][kGravLeaves];
-    __shared__ float4 hb_all[kWppWarps][kGravHits];
-    const int w = threadIdx.x >> 5;
-    int* stk = stk_all[w];
-    int* lf = lf_all[w];
-    float4* hb = hb_all[w];
-    const unsigned lane = lane_id();
-    const unsigned lt = (1u << lane) - 1u;
-    const int cnt = (int)*a.count_ptr;
-    unsigned long long c_nodes = 0, c_pairs = 0;
-    for (;;) {
-        int t = 0;
-        if (lane == 0) t = (int)atomicAdd(a.queue, 1u);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= cnt) break;
-        const int p = a.act[t];
-        const int bi = a.n_boxes == 1 ? 0 : wpp_box(a.boxes, a.n_boxes, p);
-        const BoxDesc& B = a.boxes[bi];
-        const float sf = B.sf;
-        const unsigned long long RCi = a.box_rci[bi];
-        const uint4 Xi = a.posm[p];
-        float ax = 0.f, ay = 0.f, az = 0.f, sc = 0.f;
-        int nn = 0, np = 0;
-        int sp = 0, nl = 0, nh = 0;
-        const int top = B.nlev - 1;
-        if (top == 0) {
-            nl = 1;
-            if (lane == 0) lf[0] = 0;
-        } else if (lane == 0) {
-            stk[0] = (int)((unsigned)top << 28);
-            sp = 1;
-        }
-        sp = __shfl_sync(0xffffffffu, sp, 0);
-        __syncwarp();
-        // One loop with one site for each kind of step, in this priority:
-        // evaluate 32 buffered interactions (or the last few once the walk is
-        // done), test the particles of four opened leaves (or the last few),
-        // test the children of up to four opened nodes. The buffer holds <= 31
-        // entries before a test step adds <= 32; the leaf list <= 3 before a
-        // node step adds <= 32.
-        for (;;) {
-            const bool walk_done = sp == 0 && nl == 0;
-            if (nh >= 32 || (walk_done && nh > 0)) {
-                const int k = min(nh, 32);
-                if ((int)lane < k) {
-                    const float4 h = hb[lane];
-                    const float r2 = h.x * h.x + h.y * h.y + h.z * h.z;
-                    if (r2 > 0.f) {
-                        float r;
-                        const float f = a.G * h.w * grav_K(a, r2, r);
-                        ax = fmaf(f, h.x, ax);
-                        ay = fmaf(f, h.y, ay);
-                        az = fmaf(f, h.z, az);
-                        sc = fmaf(fabsf(f), r, sc);
-                    }
-                }
-                nh -= k;   // <= 31 left: move hb[32..nh+32) down
-                const float4 v = (int)lane < nh ? hb[lane + 32] : make_float4(0.f, 0.f, 0.f, 0.f);
-                __syncwarp();
-                if ((int)lane < nh) hb[lane] = v;
-                __syncwarp();
-                continue;
-            }
-            if (walk_done) break;
-            bool take = false;
-            float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (nl >= 4 || (sp == 0 && nl > 0)) {
-                // the particles of leaves lf[0..k), lanes 8s..8s+7 on leaf s
-                const int k = min(nl, 4);
-                const int s = (int)(lane >> 3);
-                if (s < k) {
-                    const long long q = B.off + (long long)lf[s] * kLeaf + (lane & 7u);
-                    if (q < B.off + B.n && q != p) {
-                        const uint4 Xq = a.posm[q];
-                        const int dx = (int)(Xq.x - Xi.x), dy = (int)(Xq.y - Xi.y), dz = (int)(Xq.z - Xi.z);
-                        const unsigned gx = (unsigned)abs(dx) >> 8, gy = (unsigned)abs(dy) >> 8,
-                                       gz = (unsigned)abs(dz) >> 8;
-                        const unsigned long long D2 = (unsigned long long)gx * gx + (unsigned long long)gy * gy +
-                                                      (unsigned long long)gz * gz;
-                        if (D2 < RCi) {
-                            ++np;
-                            take = true;
-                            e = make_float4((float)dx * sf, (float)dy * sf, (float)dz * sf, __uint_as_float(Xq.w));
-                        }
-                    }
-                }
-                nl -= k;   // <= 31 left: move lf[k..nl+k) down
-                const int v = (int)lane < nl ? lf[lane + k] : 0;
-                __syncwarp();
-                if ((int)lane < nl) lf[lane] = v;
-            } else {
-                // the children of up to four opened nodes, one per lane
-                const int npop = sp <= 96 ? min(4, sp) : 1;
-                const int slot = (int)(lane >> 3);
-                int lev = -1, child = -1;
-                if (slot < npop) {
-                    const unsigned en = (unsigned)stk[sp - 1 - slot];
-                    const int k = (int)(en >> 28), tt = (int)(en & 0x0fffffffu);
-                    const int c = tt * kFan + (int)(lane & 7u);
-                    if (c < B.lvl_n[k - 1]) {
-                        lev = k - 1;
-                        child = c;
-                    }
-                }
-                __syncwarp();
-                sp -= npop;
-                bool push = false, leaf = false;
-                if (child >= 0) {
-                    const int nd = B.lvl_off[lev] + child;
-                    unsigned long long D2, F2, L2;
-                    grav_box(Xi, a.node_lo[nd], a.node_hi[nd], D2, F2, L2);
-                    if (D2 < RCi) {
-                        if (a.P > 0ull && D2 > 0ull && F2 < RCi && L2 <= D2 && (L2 << 16) <= a.P * D2) {
-                            ++nn;
-                            take = true;
-                            const float4 m = a.node_m[nd];
-                            const uint4 c = a.node_c[nd];
-                            e = make_float4(fmaf((float)(int)(c.x - Xi.x), sf, m.x),
-                                            fmaf((float)(int)(c.y - Xi.y), sf, m.y),
-                                            fmaf((float)(int)(c.z - Xi.z), sf, m.z), m.w);
-                        } else if (lev == 0) {
-                            leaf = true;
-                        } else {
-                            push = true;
-                        }
-                    }
-                }
-                const unsigned bp = __ballot_sync(0xffffffffu, push), bl = __ballot_sync(0xffffffffu, leaf);
-                if (push) stk[sp + __popc(bp & lt)] = (int)(((unsigned)lev << 28) | (unsigned)child);
-                if (leaf) lf[nl + __popc(bl & lt)] = child;
-                sp += __popc(bp);
-                nl += __popc(bl);
-            }
-            // append this step's interactions to the buffer
-            const unsigned bt = __ballot_sync(0xffffffffu, take);
-            if (take) hb[nh + __popc(bt & lt)] = e;
-            nh += __popc(bt);
-            __syncwarp();
-        }
-        const float fs = wpp_fold4(ax, ay, az, sc);
-        nn = warp_sum(nn);
-        np = warp_sum(np);
-        const int oi = a.perm[p];
-        if ((lane & 7u) == 0u && (lane >> 3) < 3u) a.acc[3 * (size_t)oi + (lane >> 3)] = fs;
-        if (lane == 0) {
-            if (a.n_nodes) a.n_nodes[oi] = nn;
-            if (a.n_pairs) a.n_pairs[oi] = np;
-        }
-        c_nodes += (unsigned long long)nn;
-        c_pairs += (unsigned long long)np;
-    }
-    if (lane == 0 && (c_nodes | c_pairs)) {
-        atomicAdd(&a.ctr->grav_nodes, c_nodes);
-        atomicAdd(&a.ctr->grav_pairs, c_pairs);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Shared walk for a group of up to 8 active particles of one leaf-parent node
-// ---------------------------------------------------------------------------
-//
-// The members' integer positions lie in a box G (per axis an interval of
-// span < 2^30 starting at glo). For a node, bounds over G decide it for every
-// member at once, with the per-member rule's outcome:
-//   D2_G = sum_a (gap_a(G) >> 8)^2 <= every member's D2 (the gap from the
-//          interval to the node box: 0 if they overlap, else the smaller of
-//          the ends' gaps, since a point's gap has no interior minimum off the
-//          box);
-//   F2_G = sum_a ceil(far_a(G) / 256)^2 >= every member's F2 (a point's far
-//          distance max(x - lo, hi - x), continued by gap + side off the box,
-//          is convex on any interval that does not hold the point (lo + hi)/2
-//          + 2^31 where the nearest image switches, so its largest value is at
-//          an end; an interval that holds it gets no group decision).
-// D2_G >= RCi skips the node for all; the accept test on (D2_G, F2_G) accepts
-// it for all (D2 >= D2_G and F2 <= F2_G keep every inequality, and F2 < RCi
-// implies D2 < RCi). Other nodes are decided member by member with the exact
-// rule; the members that open a node carry on with it as a member mask. A
-// particle of an opened leaf is taken for every member of the leaf's mask
-// when its largest coarse distance to the interval is inside the cutoff,
-// dropped when the smallest is not, and tested member by member otherwise.
-// Interactions are buffered with their member masks and evaluated by lanes
-// 4m..4m+3 for member m, from exact integer separations (a node entry adds
-// its centre-of-mass offset), so every count and term is the one-particle
-// kernel's.
-constexpr int kGgMembers = 8;
-
-struct GravGroupSmem {
-    int stk[kGravStack];
-    unsigned char stm[kGravStack];   // member mask of each stacked node
-    int lf[kGravLeaves];
-    unsigned short lfm[kGravLeaves]; // member mask of each opened leaf; bit 8: every particle of it
-                                     // lies inside the cutoff of every member (no tests needed)
-    uint4 hA[kGravHits];    // integer anchor (particle position or node centre), mass bits
-    float4 hB[kGravHits];   // offset from the anchor (box units: a node's centre of mass)
-    int hq[kGravHits];      // particle index (-1: a node)
-    int hm[kGravHits];      // member mask
-    uint4 mX[kGgMembers];   // member integer positions
-};
-
-// One axis of a point's exact coarse geometry against [lo, hi]: raw gap and
-// far distance (the rule of grav_axis before the coarse shift).
-__device__ __forceinline__ void grav_axis_raw(unsigned x, unsigned lo, unsigned hi, unsigned& gap, unsigned& far) {
-    if (x < lo || x > hi) {
-        gap = min(lo - x, x - hi);
-        far = gap + (hi - lo);
-    } else {
-        gap = 0u;
-        far = max(x - lo, hi - x);
-    }
-}
-
-// The group bounds of one axis (interval [e1, e1 + span]): adds to D2_G and
-// F2_G; `ok` cleared when the interval holds the switching point of the
-// nearest image, where the far bound would not hold.
-__device__ __forceinline__ void grav_axis_group(unsigned e1, unsigned span, unsigned lo, unsigned hi,
-                                                unsigned long long& D2, unsigned long long& F2, unsigned& l,
-                                                bool& ok) {
-    unsigned g1, f1, g2, f2;
-    grav_axis_raw(e1, lo, hi, g1, f1);
-    grav_axis_raw(e1 + span, lo, hi, g2, f2);
-    const bool overlap = g1 == 0u || g2 == 0u || (lo - e1) <= span;
-    const unsigned gap = overlap ? 0u : min(g1, g2);
-    const unsigned sw = lo + ((hi - lo) >> 1) + 0x80000000u;
-    if ((sw - e1) <= span) ok = false;
-    const unsigned far = max(f1, f2);
-    const unsigned g = gap >> 8, f = (unsigned)(((unsigned long long)far + 255ull) >> 8);
-    D2 += (unsigned long long)g * g;
-    F2 += (unsigned long long)f * f;
-    l = max(l, (hi - lo) >> 8);
-}
-
 // The monopole rule of the walk (see the top of the file).
 __device__ __forceinline__ bool grav_accept(unsigned long long P, unsigned long long D2, unsigned long long F2,
                                             unsigned long long L2, unsigned long long RCi) {
     return P > 0ull && D2 > 0ull && F2 < RCi && L2 <= D2 && (L2 << 16) <= P * D2;
 }
 
-// Largest and smallest coarse distance (>> 8) on one axis from x to the
-// points of the interval [e1, e1 + span] (|x - y| is convex along the
-// interval: the largest is at an end, the smallest 0 inside, else at an end).
-__device__ __forceinline__ void grav_axis_pt(unsigned x, unsigned e1, unsigned span, unsigned& hi_, unsigned& lo_) {
-    const unsigned a1 = (unsigned)abs((int)(x - e1)), a2 = (unsigned)abs((int)(x - (e1 + span)));
-    hi_ = max(a1, a2) >> 8;
-    lo_ = (x - e1) <= span ? 0u : (min(a1, a2) >> 8);
+// A node as the FP32 decision sees it, in integer units: centre and half
+// extents, and the squared bounds that settle the rule for any member.
+// With d the periodic offset of a member from the centre, the gap on an axis is
+// max(|d| - e, 0) and the far side |d| + e. Against the rule's coarse D and F
+// the FP32 norms are off by at most 2^-22 of themselves (the conversions), 2^-20
+// of the extents (through the differences), and 256 sqrt(3) + 4 units (the
+// coarse shift and the centre's half unit); the side is off by 256 units. `tol`
+// holds the extents' part and the units, the factor m the relative part.
+struct GravNode {
+    uint4 lo, hi;
+    unsigned cx, cy, cz;
+    float ex, ey, ez;
+    float out2, in2;    // D or F surely beyond the cutoff above out2, surely inside below in2
+    float acc2, opn2;   // D surely >= l / theta above acc2, surely < l / theta below opn2
+};
+
+__device__ __forceinline__ void grav_node(GravNode& N, float rcu, float inv_theta) {
+    const unsigned sx = N.hi.x - N.lo.x, sy = N.hi.y - N.lo.y, sz = N.hi.z - N.lo.z;
+    N.cx = N.lo.x + (sx >> 1);
+    N.cy = N.lo.y + (sy >> 1);
+    N.cz = N.lo.z + (sz >> 1);
+    N.ex = 0.5f * (float)sx;
+    N.ey = 0.5f * (float)sy;
+    N.ez = 0.5f * (float)sz;
+    const float m = 1.9073486328125e-06f;   // 2^-19
+    const float e = fmaxf(N.ex, fmaxf(N.ey, N.ez)), tol = fmaf(m, e, 512.f);
+    const float T = 2.f * e * inv_theta, Tl = (2.f * e - 256.f) * inv_theta;
+    const float o = rcu + tol, i = fmaxf(rcu - tol, 0.f), ah = T + tol, al = fmaxf(Tl - tol, 0.f);
+    N.out2 = o * o * (1.f + m);
+    N.in2 = i * i * (1.f - m);
+    N.acc2 = ah * ah * (1.f + m);
+    N.opn2 = al * al * (1.f - m);
 }
 
-// Error-free (TwoSum) fold of two per-lane sums over aligned quads of lanes;
-// every lane of the quad ends with both totals, rounded once.
-__device__ __forceinline__ void grav_fold_quad2(float& s1, float& s2) {
-    auto two_sum = [](float& s, float& c, float s2_, float c2_) {
-        const float t = __fadd_rn(s, s2_);
-        const float bp = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(s2_, bp));
-        s = t;
-        c = __fsub_rn(__fadd_rn(c, c2_), e);
-    };
-    float c1 = 0.f, c2 = 0.f;
-#pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
-        const float a1 = __shfl_xor_sync(0xffffffffu, s1, o), b1 = __shfl_xor_sync(0xffffffffu, c1, o);
-        const float a2 = __shfl_xor_sync(0xffffffffu, s2, o), b2 = __shfl_xor_sync(0xffffffffu, c2, o);
-        two_sum(s1, c1, a1, b1);
-        two_sum(s2, c2, a2, b2);
+constexpr int kGravSkip = 0, kGravTake = 1, kGravOpen = 2;
+
+// The rule for one member: FP32 where it is sure, the exact rule otherwise.
+__device__ __forceinline__ int grav_decide(const GravNode& N, uint4 X, unsigned long long RCi, unsigned long long P) {
+    const float dx = fabsf((float)(int)(N.cx - X.x)), dy = fabsf((float)(int)(N.cy - X.y)),
+                dz = fabsf((float)(int)(N.cz - X.z));
+    const float gx = fmaxf(dx - N.ex, 0.f), gy = fmaxf(dy - N.ey, 0.f), gz = fmaxf(dz - N.ez, 0.f);
+    const float fx = dx + N.ex, fy = dy + N.ey, fz = dz + N.ez;
+    const float D2f = fmaf(gx, gx, fmaf(gy, gy, gz * gz)), F2f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+    if (D2f > N.out2) return kGravSkip;
+    if (D2f < N.in2) {
+        if (P == 0ull || F2f > N.out2 || D2f < N.opn2) return kGravOpen;
+        if (F2f < N.in2 && D2f > N.acc2) return kGravTake;
     }
-    s1 = __fsub_rn(s1, c1);
-    s2 = __fsub_rn(s2, c2);
+    unsigned long long D2, F2, L2;
+    grav_box(X, N.lo, N.hi, D2, F2, L2);
+    return D2 >= RCi ? kGravSkip : grav_accept(P, D2, F2, L2, RCi) ? kGravTake : kGravOpen;
 }
 
-__global__ void __launch_bounds__(kWppThreads) k_gravity_group(GravArgs a) {
-    __shared__ GravGroupSmem smem[kWppWarps];
-    GravGroupSmem& sm = smem[threadIdx.x >> 5];
+// Error-free (TwoSum) fold of a per-lane sum over aligned runs of W lanes; every
+// lane of a run ends with the total, rounded once.
+template <int W>
+__device__ __forceinline__ float grav_fold(float s) {
+    float c = 0.f;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) {
+        const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+        const float t = __fadd_rn(s, s2);
+        const float bp = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(s2, bp));
+        s = t;
+        c = __fsub_rn(__fadd_rn(c, c2), e);
+    }
+    return __fsub_rn(s, c);
+}
+
+template <int M>
+struct GravSmem {
+    int stk[kGravStack];
+    unsigned char stm[kGravStack];   // member mask of each stacked node
+    uint4 mX[M];                     // member integer positions
+    int lf[M][kGravLeaves];          // opened leaves (first particle)
+    int nd[M][kGravNodes];           // accepted nodes (global index)
+};
+
+template <int M>
+__global__ void __launch_bounds__(kWppThreads, 5) k_gravity(GravArgs a) {
+    __shared__ GravSmem<M> smem[kWppWarps];
+    GravSmem<M>& sm = smem[threadIdx.x >> 5];
+    constexpr int W = 32 / M;   // lanes per member
     const unsigned lane = lane_id();
     const unsigned lt = (1u << lane) - 1u;
     const int cnt = (int)*a.count_ptr;
-    const int mm = (int)(lane >> 2), sub = (int)(lane & 3u);   // evaluation: lane (member, quarter)
+    const int mm = (int)lane / W, sub = (int)lane % W;   // list work: lane (member, part)
     unsigned long long c_nodes = 0, c_pairs = 0;
     for (;;) {
         int t0 = 0;
-        if (lane == 0) t0 = (int)atomicAdd(a.queue, (unsigned)kGgMembers);
+        if (lane == 0) t0 = (int)atomicAdd(a.queue, (unsigned)M);
         t0 = __shfl_sync(0xffffffffu, t0, 0);
         if (t0 >= cnt) break;
-        const int t1 = min(t0 + kGgMembers, cnt);
+        const int t1 = min(t0 + M, cnt);
         for (int t = t0; t < t1;) {
             const WppGroup G = wpp_group(a.boxes, a.n_boxes, a.act, t, t1, 6);
             t += G.n;
             const BoxDesc& B = a.boxes[G.box];
             const float sf = B.sf;
-            const unsigned long long RCi = a.box_rci[G.box];
-            const unsigned full = (1u << G.n) - 1u;
-            // members: lane l < G.n holds member l; the group's interval per axis
+            const GravBox gb = a.gbox[G.box];
+            const int off = (int)B.off, pend = (int)(B.off + B.n);
             uint4 Xl = make_uint4(0u, 0u, 0u, 0u);
             if (G.p >= 0) Xl = a.posm[G.p];
-            if ((int)lane < kGgMembers) sm.mX[lane] = Xl;
-            const unsigned X0x = __shfl_sync(0xffffffffu, Xl.x, 0), X0y = __shfl_sync(0xffffffffu, Xl.y, 0),
-                           X0z = __shfl_sync(0xffffffffu, Xl.z, 0);
-            const bool mv = G.p >= 0;
-            const int dx0 = mv ? (int)(Xl.x - X0x) : 0, dy0 = mv ? (int)(Xl.y - X0y) : 0,
-                      dz0 = mv ? (int)(Xl.z - X0z) : 0;
-            const int lox = warp_min(dx0), loy = warp_min(dy0), loz = warp_min(dz0);
-            const long long sxl = (long long)warp_max(dx0) - lox, syl = (long long)warp_max(dy0) - loy,
-                            szl = (long long)warp_max(dz0) - loz;
-            // a group spanning a quarter of the box or more takes no group decision
-            const bool gok = sxl < (1ll << 30) && syl < (1ll << 30) && szl < (1ll << 30);
-            const unsigned gex = X0x + (unsigned)lox, gey = X0y + (unsigned)loy, gez = X0z + (unsigned)loz;
-            const unsigned spx = (unsigned)sxl, spy = (unsigned)syl, spz = (unsigned)szl;
-            // the evaluation lanes' member
+            if ((int)lane < M) sm.mX[lane] = Xl;
             const uint4 Xm = make_uint4(__shfl_sync(0xffffffffu, Xl.x, mm), __shfl_sync(0xffffffffu, Xl.y, mm),
                                         __shfl_sync(0xffffffffu, Xl.z, mm), 0u);
             const int pmm = __shfl_sync(0xffffffffu, G.p, mm);
-            const bool mlive = mm < G.n;
-            float ax = 0.f, ay = 0.f, az = 0.f, sc = 0.f;
+            float2 ax = both(0.f), ay = ax, az = ax;   // this list's sums
+            float Sx = 0.f, Sy = 0.f, Sz = 0.f, Cx = 0.f, Cy = 0.f, Cz = 0.f;   // the lists' (Kahan)
             int nn = 0, np = 0;
-            int sp = 0, nl = 0, nh = 0;
+            int nl[M], na[M];   // list lengths (warp-uniform)
+#pragma unroll
+            for (int m = 0; m < M; ++m) nl[m] = na[m] = 0;
+            int sp = 0;
             const int top = B.nlev - 1;
-            if (top == 0) {
-                nl = 1;
-                if (lane == 0) {
-                    sm.lf[0] = 0;
-                    sm.lfm[0] = (unsigned short)full;
-                }
+            if (lane == 0) {
+                sm.stk[0] = (int)((unsigned)top << 28);
+                sm.stm[0] = (unsigned char)((1u << G.n) - 1u);
+            }
+            if (top == 0) {   // a single leaf: opened whatever the rule says
+                if ((int)lane < M) sm.lf[lane][0] = off;
+#pragma unroll
+                for (int m = 0; m < M; ++m) nl[m] = m < G.n ? 1 : 0;
             } else {
-                if (lane == 0) {
-                    sm.stk[0] = (int)((unsigned)top << 28);
-                    sm.stm[0] = (unsigned char)full;
-                }
                 sp = 1;
             }
             __syncwarp();
-            // The one-particle kernel's loop: evaluate 32 buffered interactions (or
-            // the last few once the walk is done), test the particles of four
-            // opened leaves (or the last few), test the children of up to four
-            // opened nodes; with a member mask on every node, leaf and entry.
+            // two interactions; ok false: none
+            auto add = [&](float2 ex, float2 ey, float2 ez, float2 r2, float2 m, bool ok0, bool ok1) {
+                ok0 = ok0 && r2.x > 0.f;   // coincident: no force
+                ok1 = ok1 && r2.y > 0.f;
+                if (!ok0 && !ok1) return;
+                m = mul2(both(a.G), make_float2(ok0 ? m.x : 0.f, ok1 ? m.y : 0.f));
+                const float2 f = mul2(m, grav_K(a, make_float2(ok0 ? r2.x : 1.f, ok1 ? r2.y : 1.f)));
+                ax = fma2(f, ex, ax);
+                ay = fma2(f, ey, ay);
+                az = fma2(f, ez, az);
+            };
+            // a particle that passed neither FP32 bound: the exact test
+            auto inside = [&](uint4 X) {
+                const unsigned gx = (unsigned)abs((int)(X.x - Xm.x)) >> 8, gy = (unsigned)abs((int)(X.y - Xm.y)) >> 8,
+                               gz = (unsigned)abs((int)(X.z - Xm.z)) >> 8;
+                return (unsigned long long)gx * gx + (unsigned long long)gy * gy + (unsigned long long)gz * gz < gb.RCi;
+            };
+            auto total = [&]() {
+                kahan_add(Sx, Cx, ax.x + ax.y);
+                kahan_add(Sy, Cy, ay.x + ay.y);
+                kahan_add(Sz, Cz, az.x + az.y);
+                ax = ay = az = both(0.f);
+            };
+            bool done = sp == 0;
             for (;;) {
-                const bool walk_done = sp == 0 && nl == 0;
-                if (nh >= 32 || (walk_done && nh > 0)) {
-                    const int k = min(nh, 32);
-#pragma unroll 2
-                    for (int jj = 0; jj < 8; ++jj) {
-                        const int c = sub + 4 * jj;
-                        if (c < k && mlive && ((sm.hm[c] >> mm) & 1) && sm.hq[c] != pmm) {
-                            const uint4 A = sm.hA[c];
-                            const float4 Bo = sm.hB[c];
-                            if (sm.hq[c] < 0) ++nn; else ++np;
-                            const float ex = fmaf((float)(int)(A.x - Xm.x), sf, Bo.x),
-                                        ey = fmaf((float)(int)(A.y - Xm.y), sf, Bo.y),
-                                        ez = fmaf((float)(int)(A.z - Xm.z), sf, Bo.z);
-                            const float r2 = ex * ex + ey * ey + ez * ez;
-                            if (r2 > 0.f) {
-                                float r;
-                                const float f = a.G * __uint_as_float(A.w) * grav_K(a, r2, r);
-                                ax = fmaf(f, ex, ax);
-                                ay = fmaf(f, ey, ay);
-                                az = fmaf(f, ez, az);
-                                sc = fmaf(fabsf(f), r, sc);
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    nh -= k;   // <= 31 left: move entries [32, nh + 32) down
-                    uint4 vA = make_uint4(0u, 0u, 0u, 0u);
-                    float4 vB = make_float4(0.f, 0.f, 0.f, 0.f);
-                    int vq = 0, vm = 0;
-                    if ((int)lane < nh) {
-                        vA = sm.hA[lane + 32];
-                        vB = sm.hB[lane + 32];
-                        vq = sm.hq[lane + 32];
-                        vm = sm.hm[lane + 32];
-                    }
-                    __syncwarp();
-                    if ((int)lane < nh) {
-                        sm.hA[lane] = vA;
-                        sm.hB[lane] = vB;
-                        sm.hq[lane] = vq;
-                        sm.hm[lane] = vm;
-                    }
-                    __syncwarp();
-                    continue;
+                int ml = 0, mn = 0;
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    ml = max(ml, nl[m]);
+                    mn = max(mn, na[m]);
                 }
-                if (walk_done) break;
-                unsigned emask = 0u;   // members taking this lane's interaction
-                uint4 eA = make_uint4(0u, 0u, 0u, 0u);
-                float4 eB = make_float4(0.f, 0.f, 0.f, 0.f);
-                int eq = -1;
-                if (nl >= 4 || (sp == 0 && nl > 0)) {
-                    // the particles of leaves lf[0..k), lanes 8s..8s+7 on leaf s
-                    const int k = min(nl, 4);
-                    const int s = (int)(lane >> 3);
-                    if (s < k) {
-                        const unsigned M = sm.lfm[s] & 0xffu;
-                        const bool allin = (sm.lfm[s] >> 8) != 0u;
-                        const long long q = B.off + (long long)sm.lf[s] * kLeaf + (lane & 7u);
-                        if (q < B.off + B.n) {
-                            const uint4 Xq = a.posm[q];
-                            bool decided = false;
-                            if (allin) {
-                                decided = true;
-                                emask = M;
-                            } else if (gok) {
-                                unsigned hx, lx, hy, ly, hz, lz;
-                                grav_axis_pt(Xq.x, gex, spx, hx, lx);
-                                grav_axis_pt(Xq.y, gey, spy, hy, ly);
-                                grav_axis_pt(Xq.z, gez, spz, hz, lz);
-                                const unsigned long long U = (unsigned long long)hx * hx +
-                                                             (unsigned long long)hy * hy +
-                                                             (unsigned long long)hz * hz;
-                                const unsigned long long Lw = (unsigned long long)lx * lx +
-                                                              (unsigned long long)ly * ly +
-                                                              (unsigned long long)lz * lz;
-                                if (Lw >= RCi) {
-                                    decided = true;
-                                } else if (U < RCi) {
-                                    decided = true;
-                                    emask = M;
-                                }
-                            }
-                            if (!decided) {
-                                for (unsigned r = M; r; r &= r - 1u) {
-                                    const int m = __ffs(r) - 1;
-                                    const uint4 Y = sm.mX[m];
-                                    const unsigned gx = (unsigned)abs((int)(Xq.x - Y.x)) >> 8,
-                                                   gy = (unsigned)abs((int)(Xq.y - Y.y)) >> 8,
-                                                   gz = (unsigned)abs((int)(Xq.z - Y.z)) >> 8;
-                                    const unsigned long long D2 = (unsigned long long)gx * gx +
-                                                                  (unsigned long long)gy * gy +
-                                                                  (unsigned long long)gz * gz;
-                                    if (D2 < RCi) emask |= 1u << m;
-                                }
-                            }
-                            eA = Xq;
-                            eq = (int)q;
-                        }
+                if (done ? ml > 0 : ml > kGravLeaves - 32) {
+                    // the particles of the opened leaves, two per lane and step, the
+                    // next step's positions loaded ahead
+                    int k = 0;
+#pragma unroll
+                    for (int m = 0; m < M; ++m) {
+                        k = mm == m ? nl[m] : k;
+                        nl[m] = 0;
                     }
-                    nl -= k;   // <= 31 left: move lf[k..nl+k) down
-                    const int v = (int)lane < nl ? sm.lf[lane + k] : 0;
-                    const unsigned short vm = (int)lane < nl ? sm.lfm[lane + k] : (unsigned short)0;
+                    const int* lf = sm.lf[mm];
+                    k *= kLeaf;
+                    // (the last leaf may reach past the box: those reads stay in the padded store)
+                    auto fetch = [&](int j, uint4& X) {
+                        const int q = j < k ? lf[j >> 3] + (j & 7) : pend;
+                        X = a.posm[j < k ? q : off];
+                        return q < pend;
+                    };
+                    uint4 n0, n1;
+                    bool v0 = fetch(sub, n0), v1 = fetch(sub + W, n1);
+                    for (int j = sub; j < k; j += 2 * W) {
+                        const uint4 X0 = n0, X1 = n1;
+                        bool i0 = v0, i1 = v1;
+                        v0 = fetch(j + 2 * W, n0);
+                        v1 = fetch(j + 3 * W, n1);
+                        const float2 s2 = both(sf);
+                        const float2 ex = mul2(make_float2((float)(int)(X0.x - Xm.x), (float)(int)(X1.x - Xm.x)), s2),
+                                     ey = mul2(make_float2((float)(int)(X0.y - Xm.y), (float)(int)(X1.y - Xm.y)), s2),
+                                     ez = mul2(make_float2((float)(int)(X0.z - Xm.z), (float)(int)(X1.z - Xm.z)), s2);
+                        const float2 r2 = fma2(ez, ez, fma2(ey, ey, mul2(ex, ex)));
+                        i0 = i0 && !(r2.x > gb.r2_out);
+                        i1 = i1 && !(r2.y > gb.r2_out);
+                        if (i0 && !(r2.x < gb.r2_in)) i0 = inside(X0);
+                        if (i1 && !(r2.y < gb.r2_in)) i1 = inside(X1);
+                        np += (i0 ? 1 : 0) + (i1 ? 1 : 0);
+                        add(ex, ey, ez, r2, make_float2(__uint_as_float(X0.w), __uint_as_float(X1.w)), i0, i1);
+                    }
+                    total();
                     __syncwarp();
-                    if ((int)lane < nl) {
-                        sm.lf[lane] = v;
-                        sm.lfm[lane] = vm;
+                }
+                if (done ? mn > 0 : mn > kGravNodes - 32) {
+                    int k = 0;
+#pragma unroll
+                    for (int m = 0; m < M; ++m) {
+                        k = mm == m ? na[m] : k;
+                        na[m] = 0;
                     }
-                } else {
-                    // the children of up to four opened nodes, one per lane
-                    const int npop = sp <= 96 ? min(4, sp) : 1;
-                    const int slot = (int)(lane >> 3);
-                    int lev = -1, child = -1;
-                    unsigned M = 0u;
-                    if (slot < npop) {
-                        const unsigned en = (unsigned)sm.stk[sp - 1 - slot];
-                        M = sm.stm[sp - 1 - slot];
-                        const int k = (int)(en >> 28), tt = (int)(en & 0x0fffffffu);
-                        const int c = tt * kFan + (int)(lane & 7u);
-                        if (c < B.lvl_n[k - 1]) {
-                            lev = k - 1;
-                            child = c;
-                        }
+                    nn += k;
+                    const int* nd = sm.nd[mm];
+                    for (int j = sub; j < k; j += 2 * W) {
+                        const bool two = j + W < k;
+                        const int i0 = nd[j], i1 = nd[two ? j + W : j];
+                        const uint4 C0 = a.node_c[i0], C1 = a.node_c[i1];
+                        const float4 q0 = a.node_m[i0], q1 = a.node_m[i1];
+                        const float2 s2 = both(sf);
+                        const float2 ex = fma2(make_float2((float)(int)(C0.x - Xm.x), (float)(int)(C1.x - Xm.x)), s2,
+                                               make_float2(q0.x, q1.x)),
+                                     ey = fma2(make_float2((float)(int)(C0.y - Xm.y), (float)(int)(C1.y - Xm.y)), s2,
+                                               make_float2(q0.y, q1.y)),
+                                     ez = fma2(make_float2((float)(int)(C0.z - Xm.z), (float)(int)(C1.z - Xm.z)), s2,
+                                               make_float2(q0.z, q1.z));
+                        add(ex, ey, ez, fma2(ez, ez, fma2(ey, ey, mul2(ex, ex))), make_float2(q0.w, q1.w), true, two);
                     }
+                    total();
                     __syncwarp();
-                    sp -= npop;
-                    unsigned om = 0u;   // members that open the child
-                    bool allin = false; // an opened leaf wholly inside every member's cutoff
-                    if (child >= 0) {
-                        const int nd = B.lvl_off[lev] + child;
-                        const uint4 lo = a.node_lo[nd], hi = a.node_hi[nd];
-                        bool decided = false;
-                        if (gok) {
-                            unsigned long long D2 = 0ull, F2 = 0ull;
-                            unsigned l = 0u;
-                            bool ok = true;
-                            grav_axis_group(gex, spx, lo.x, hi.x, D2, F2, l, ok);
-                            grav_axis_group(gey, spy, lo.y, hi.y, D2, F2, l, ok);
-                            grav_axis_group(gez, spz, lo.z, hi.z, D2, F2, l, ok);
-                            if (D2 >= RCi) {
-                                decided = true;
-                            } else if (ok && grav_accept(a.P, D2, F2, (unsigned long long)l * l, RCi)) {
-                                decided = true;
-                                emask = M;
-                            }
-                            // a point of the box is no farther from a member than the box's
-                            // far side, so F2_G < RCi puts every particle inside the cutoff
-                            allin = ok && F2 < RCi;
-                        }
-                        if (!decided) {
-                            for (unsigned r = M; r; r &= r - 1u) {
-                                const int m = __ffs(r) - 1;
-                                unsigned long long D2, F2, L2;
-                                grav_box(sm.mX[m], lo, hi, D2, F2, L2);
-                                if (D2 < RCi) {
-                                    if (grav_accept(a.P, D2, F2, L2, RCi)) emask |= 1u << m;
-                                    else om |= 1u << m;
-                                }
-                            }
-                        }
-                        if (emask) {
-                            const float4 nm = a.node_m[nd];
-                            eA = a.node_c[nd];
-                            eA.w = __float_as_uint(nm.w);
-                            eB = make_float4(nm.x, nm.y, nm.z, 0.f);
-                        }
-                    }
-                    const bool push = om != 0u && lev > 0, leaf = om != 0u && lev == 0;
-                    const unsigned bp = __ballot_sync(0xffffffffu, push), bl = __ballot_sync(0xffffffffu, leaf);
-                    if (push) {
-                        const int o = sp + __popc(bp & lt);
-                        sm.stk[o] = (int)(((unsigned)lev << 28) | (unsigned)child);
-                        sm.stm[o] = (unsigned char)om;
-                    }
-                    if (leaf) {
-                        const int o = nl + __popc(bl & lt);
-                        sm.lf[o] = child;
-                        sm.lfm[o] = (unsigned short)(om | (allin ? 0x100u : 0u));
-                    }
-                    sp += __popc(bp);
-                    nl += __popc(bl);
                 }
-                // append this step's interactions to the buffer
-                const bool take = emask != 0u;
-                const unsigned bt = __ballot_sync(0xffffffffu, take);
-                if (take) {
-                    const int o = nh + __popc(bt & lt);
-                    sm.hA[o] = eA;
-                    sm.hB[o] = eB;
-                    sm.hq[o] = eq;
-                    sm.hm[o] = (int)emask;
+                if (done) break;
+                // the children of up to four opened nodes, one per lane
+                const int npop = sp <= 96 ? min(4, sp) : 1;
+                const int slot = (int)(lane >> 3);
+                int lev = -1, child = -1;
+                unsigned mask = 0u;
+                if (slot < npop) {
+                    const unsigned en = (unsigned)sm.stk[sp - 1 - slot];
+                    const int k = (int)(en >> 28), c = (int)(en & 0x0fffffffu) * kFan + (int)(lane & 7u);
+                    if (c < B.lvl_n[k - 1]) {
+                        lev = k - 1;
+                        child = c;
+                        mask = sm.stm[sp - 1 - slot];
+                    }
                 }
-                nh += __popc(bt);
+                __syncwarp();
+                sp -= npop;
+                const int id = B.lvl_off[max(lev, 0)] + max(child, 0);
+                GravNode N;
+                N.lo = a.node_lo[id];
+                N.hi = a.node_hi[id];
+                grav_node(N, gb.rcu, a.inv_theta);
+                unsigned om = 0u;   // members that open the child
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    int v = kGravSkip;
+                    if ((mask >> m) & 1u) v = grav_decide(N, sm.mX[m], gb.RCi, a.P);
+                    if (v == kGravOpen) om |= 1u << m;
+                    const unsigned bl = __ballot_sync(0xffffffffu, v == kGravOpen && lev == 0),
+                                   bn = __ballot_sync(0xffffffffu, v == kGravTake);
+                    if (v == kGravOpen && lev == 0) sm.lf[m][nl[m] + __popc(bl & lt)] = off + child * kLeaf;
+                    if (v == kGravTake) sm.nd[m][na[m] + __popc(bn & lt)] = id;
+                    nl[m] += __popc(bl);
+                    na[m] += __popc(bn);
+                }
+                const bool push = om != 0u && lev > 0;
+                const unsigned bp = __ballot_sync(0xffffffffu, push);
+                if (push) {
+                    const int o = sp + __popc(bp & lt);
+                    sm.stk[o] = (int)(((unsigned)lev << 28) | (unsigned)child);
+                    sm.stm[o] = (unsigned char)om;
+                }
+                sp += __popc(bp);
+                done = sp == 0;
                 __syncwarp();
             }
-            // per member: fold its quad's sums, write its outputs
-            grav_fold_quad2(ax, ay);
-            grav_fold_quad2(az, sc);
-            nn += __shfl_xor_sync(0xffffffffu, nn, 1);
-            nn += __shfl_xor_sync(0xffffffffu, nn, 2);
-            np += __shfl_xor_sync(0xffffffffu, np, 1);
-            np += __shfl_xor_sync(0xffffffffu, np, 2);
-            if (mlive) {
+            // per member: fold its lanes' sums, write its outputs
+            Sx = grav_fold<W>(Sx - Cx);
+            Sy = grav_fold<W>(Sy - Cy);
+            Sz = grav_fold<W>(Sz - Cz);
+#pragma unroll
+            for (int o = 1; o < W; o <<= 1) np += __shfl_xor_sync(0xffffffffu, np, o);
+            if (mm < G.n && sub == 0) {
+                np -= gb.RCi > 0ull ? 1 : 0;   // itself: in its own leaf, always opened, at distance 0
                 const int oi = a.perm[pmm];
-                if (sub < 3) a.acc[3 * (size_t)oi + sub] = sub == 0 ? ax : (sub == 1 ? ay : az);
-                if (sub == 3) {
-                    if (a.n_nodes) a.n_nodes[oi] = nn;
-                    if (a.n_pairs) a.n_pairs[oi] = np;
-                }
-                if (sub == 0) {
-                    c_nodes += (unsigned long long)nn;
-                    c_pairs += (unsigned long long)np;
-                }
+                a.acc[3 * (size_t)oi] = Sx;
+                a.acc[3 * (size_t)oi + 1] = Sy;
+                a.acc[3 * (size_t)oi + 2] = Sz;
+                if (a.n_nodes) a.n_nodes[oi] = nn;
+                if (a.n_pairs) a.n_pairs[oi] = np;
+                c_nodes += (unsigned long long)nn;
+                c_pairs += (unsigned long long)np;
             }
             __syncwarp();
         }
@@ -738,18 +563,25 @@ __global__ void __launch_bounds__(kWppThreads) k_gravity_group(GravArgs a) {
     }
 }
 
+template <int M>
+static void grav_run(sph_ctx* ctx, const GravArgs& a, int64_t n_active, cudaStream_t s) {
+    const long long want = (n_active + M * kWppWarps - 1) / (M * kWppWarps);
+    const int blocks = (int)std::max<long long>(1, std::min<long long>((long long)ctx->sm_count * 8, want));
+    k_gravity<M><<<blocks, kWppThreads, 0, s>>>(a);
+}
+
 cudaError_t launch_gravity(sph_ctx* ctx, const GravityLaunch& L, int64_t n_active, cudaStream_t s) {
     sph_grid* g = const_cast<sph_grid*>(L.g);
     const int nb = g->n_boxes;
-    dim3 lg((g->max_leaves + 127) / 128, nb);
-    k_grav_leaf_moments<<<lg, 128, 0, s>>>(g->posm, g->boxes, g->node_c, g->node_m);
+    k_grav_low<<<dim3((g->max_leaves + kTreeT - 1) / kTreeT, nb), kTreeT, 0, s>>>(g->posm, g->boxes, g->node_c,
+                                                                              g->node_m);
     ++ctx->launches;
-    for (int lev = 1; lev < g->max_lev; ++lev) {
-        dim3 ng((g->lvl_max[lev] + 127) / 128, nb);
-        k_grav_node_moments<<<ng, 128, 0, s>>>(lev, g->boxes, g->node_c, g->node_m);
+    if (g->max_lev > kTreeLow) {
+        k_grav_top<<<nb, kTreeTopT, 0, s>>>(g->boxes, g->node_c, g->node_m);
         ++ctx->launches;
     }
-    k_grav_box_rc<<<(nb + 127) / 128, 128, 0, s>>>(g->boxes, nb, L.r_cut, g->box_rci);
+    GravBox* gbox = reinterpret_cast<GravBox*>(g->grav_box);
+    k_grav_box_rc<<<(nb + 127) / 128, 128, 0, s>>>(g->boxes, nb, L.r_cut, gbox);
     ++ctx->launches;
     cudaError_t e = cudaMemsetAsync(ctx->queue + 4, 0, sizeof(unsigned), s);
     if (e) return e;
@@ -765,26 +597,29 @@ cudaError_t launch_gravity(sph_ctx* ctx, const GravityLaunch& L, int64_t n_activ
     a.node_hi = g->node_hi;
     a.node_c = g->node_c;
     a.node_m = g->node_m;
-    a.box_rci = g->box_rci;
+    a.gbox = gbox;
     a.acc = L.acc;
     a.n_nodes = L.n_nodes;
     a.n_pairs = L.n_pairs;
     a.ctr = ctx->counters;
     a.G = (float)L.G;
     a.P = (unsigned long long)std::rint(L.theta * L.theta * 65536.0);
+    a.inv_theta = a.P ? (float)(256.0 / std::sqrt((double)a.P)) : 0.f;
     a.hs = (float)L.h_soft;
     a.inv_hs = L.h_soft > 0.0 ? (float)(1.0 / L.h_soft) : 0.f;
     a.inv2rs = L.r_split > 0.0 ? (float)(0.5 / L.r_split) : 0.f;
-    if (wpp_groups_pay(ctx, n_active, g->n)) {
-        // groups of up to 8 particles of a leaf-parent node share one walk
-        const long long want = (n_active + kGgMembers * kWppWarps - 1) / (kGgMembers * kWppWarps);
-        const int blocks = (int)std::max<long long>(1, std::min<long long>((long long)ctx->sm_count * 8, want));
-        k_gravity_group<<<blocks, kWppThreads, 0, s>>>(a);
-    } else {
-        const long long want = (n_active + kWppWarps - 1) / kWppWarps;
-        const int blocks = (int)std::max<long long>(1, std::min<long long>((long long)ctx->sm_count * 8, want));
-        k_gravity<<<blocks, kWppThreads, 0, s>>>(a);
-    }
+    // Members per walk: more of them share the node loads and tests, but a group
+    // of 8 takes 8 times as long, so a set must be large enough to fill the GPU
+    // with groups several times over, and dense enough that groups are full.
+    // Measured (clustered, theta 0.5), us for 1/2/4/8 members: 9,000 of 30,000 active
+    // 139/170/209/430; all of 30,000 280/253/267/320; of 60,000 559/493/478/531;
+    // of 500,000 5255/4514/4108/4078; of 1M 12700/11200/10440/10100; 100,000 of 1M
+    // 1588/1484/1524/1956; 25,000 of 500,000 396/407/467/904.
+    const long long sm = ctx->sm_count, na = n_active, n = g->n;
+    if (na >= 3000 * sm && na * 2 >= n) grav_run<8>(ctx, a, na, s);
+    else if (na >= 320 * sm && na * 4 >= n) grav_run<4>(ctx, a, na, s);
+    else if (na >= 176 * sm && na * 16 >= n) grav_run<2>(ctx, a, na, s);
+    else grav_run<1>(ctx, a, na, s);
     ++ctx->launches;
     return cudaGetLastError();
 }

@@ -625,7 +625,7 @@ void grid_free(sph_grid* g) {
     void* ptrs[] = {g->boxes, g->posm, g->xq, g->perm, g->rank, g->keys, g->node_lo, g->node_hi,
                     g->node_hmax, g->act, g->flag, g->scan, g->scan_tmp, g->list_a, g->list_b, g->st_lo, g->st_hi, g->list_n, g->d_off, g->d_L,
                     g->k2, g->v2, g->rs_work, g->node_c, g->node_e, g->posf,
-                    g->fvel, g->fthermo, g->fposh, g->fvm, g->fbal, g->fcond, g->fvisc, g->node_m, g->box_rci, g->nbr, g->nbr_off, g->nbr_n, g->ext_n, g->ext, g->list_xh, g->list_st, g->fb_list, g->list_ep, g->mp_x, g->bw_ga, g->bw_xbar, g->bw_rd, g->bw_f, g->mp_j, g->den_left};
+                    g->fvel, g->fthermo, g->fposh, g->fvm, g->fbal, g->fcond, g->fvisc, g->node_m, g->grav_box, g->nbr, g->nbr_off, g->nbr_n, g->ext_n, g->ext, g->list_xh, g->list_st, g->fb_list, g->list_ep, g->mp_x, g->bw_ga, g->bw_xbar, g->bw_rd, g->bw_f, g->mp_j, g->den_left};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete g;
@@ -684,7 +684,6 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
             if (lev >= kMaxLev) { ctx->err = "box too large for the hierarchy"; delete g; return SPH_ERR_INVALID; }
             B.lvl_off[lev] = node;
             B.lvl_n[lev] = cnt;
-            g->lvl_max[lev] = std::max(g->lvl_max[lev], cnt);
             node += cnt;
             ++lev;
             if (cnt == 1) break;
@@ -719,7 +718,8 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
         GRID_CHECK(cudaMemcpyAsync(g->d_L, Ls, sizeof(double) * nb, cudaMemcpyHostToDevice, s));
         GRID_CHECK(cudaStreamSynchronize(s));  // host staging buffers go out of scope
     }
-    GRID_CHECK(cudaMalloc(&g->posm, sizeof(uint4) * n));
+    // (padded: the gravity kernel reads whole leaves, the last one past its end)
+    GRID_CHECK(cudaMalloc(&g->posm, sizeof(uint4) * ((size_t)n + kLeaf)));
     GRID_CHECK(cudaMalloc(&g->xq, sizeof(uint4) * n));
     GRID_CHECK(cudaMalloc(&g->perm, sizeof(int32_t) * n));
     GRID_CHECK(cudaMalloc(&g->rank, sizeof(int32_t) * n));
@@ -739,7 +739,7 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
     GRID_CHECK(cudaMalloc(&g->fcond, sizeof(float2) * n));
     GRID_CHECK(cudaMalloc(&g->fvisc, sizeof(float2) * n));
     GRID_CHECK(cudaMalloc(&g->node_m, sizeof(float4) * node));
-    GRID_CHECK(cudaMalloc(&g->box_rci, sizeof(unsigned long long) * nb));
+    GRID_CHECK(cudaMalloc(&g->grav_box, (size_t)kGravBoxBytes * nb));
     // the near-list indices of the density pass's member-parallel path, one
     // block of kMpMembers x kMpCap per persistent warp
     GRID_CHECK(cudaMalloc(&g->mp_j, sizeof(int32_t) * (size_t)ctx->sm_count * kMpWarpsPerSm * kMpMembers * kMpCap));

@@ -33,7 +33,6 @@ struct sph_grid {
     int n_nodes = 0;
     int max_leaves = 0;                    // max over boxes of level-0 nodes
     int max_lev = 0;                       // max over boxes of the level count
-    int lvl_max[sph::kMaxLev] = {};        // max over boxes of the nodes on each level
     std::vector<sph::BoxDesc> boxes_h;
     sph::BoxDesc* boxes = nullptr;         // device
     uint4* posm = nullptr;                 // sorted: X, Y, Z, mass bits
@@ -55,7 +54,7 @@ struct sph_grid {
     float2* fcond = nullptr;               // per force call with conduction, sorted: u, kappa
     float2* fvisc = nullptr;               // per force call with per-particle viscosity, sorted: factor, alpha
     float4* node_m = nullptr;              // per gravity call, per node: centre of mass - node centre, mass
-    unsigned long long* box_rci = nullptr; // per gravity call, per box: coarse squared cutoff
+    unsigned char* grav_box = nullptr;     // per gravity call, per box: the cutoff (kGravBoxBytes each)
     // per-call scratch, sized at build so that calls never allocate
     int32_t* act = nullptr;                // active particles, sorted indices, sorted order
     uint8_t* flag = nullptr;               // n
@@ -103,6 +102,7 @@ struct sph_grid {
 namespace sph {
 
 constexpr int kQueues = 8;
+constexpr int kGravBoxBytes = 24;
 constexpr int kListPool = 128;  // neighbour-list pool entries per particle (lists vary in length)
 constexpr int kExtCap = 128;    // extra-partner segment per particle (262k clustered: mean 24, max 106)
 constexpr unsigned kExtUnusable = 0xffffffffu;
