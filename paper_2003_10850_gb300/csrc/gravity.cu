@@ -589,7 +589,7 @@ cudaError_t launch_gravity(sph_ctx* ctx, const GravityLaunch& L, int64_t n_activ
     a.boxes = g->boxes;
     a.n_boxes = nb;
     a.act = g->act;
-    a.count_ptr = g->scan + g->n;
+    a.count_ptr = g->act_n;
     a.queue = ctx->queue + 4;
     a.posm = g->posm;
     a.perm = g->perm;

@@ -85,103 +85,6 @@ __global__ void k_quantize(const P* __restrict__ pos, const float* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan (reduce, scan the block sums, apply), 4096 items per block
-// ---------------------------------------------------------------------------
-
-constexpr int kScanT = 1024, kScanIPT = 4, kScanTile = kScanT * kScanIPT;
-
-__device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* sm, unsigned& total) {
-    // sm: 32 words. Returns the exclusive prefix of v over the block.
-    unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    unsigned x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= (unsigned)o) x += y;
-    }
-    if (lane == 31) sm[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        unsigned nw = blockDim.x >> 5;
-        unsigned w = lane < nw ? sm[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= (unsigned)o) w += y;
-        }
-        sm[lane] = w;  // inclusive warp totals
-    }
-    __syncthreads();
-    total = sm[(blockDim.x >> 5) - 1];
-    unsigned before = warp ? sm[warp - 1] : 0u;
-    unsigned r = before + x - v;
-    __syncthreads();
-    return r;
-}
-
-template <typename In>
-__global__ void k_scan_reduce(const In* __restrict__ in, int n, unsigned* __restrict__ bsum) {
-    __shared__ unsigned sm[32];
-    int base = blockIdx.x * kScanTile + threadIdx.x * kScanIPT;
-    unsigned s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanIPT; ++k)
-        if (base + k < n) s += (unsigned)in[base + k];
-    unsigned tot;
-    block_excl_scan(s, sm, tot);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
-}
-
-__global__ void k_scan_bsums(unsigned* bsum, int nb) {
-    __shared__ unsigned sm[32];
-    unsigned carry = 0;
-    for (int base = 0; base < nb; base += blockDim.x) {
-        int i = base + threadIdx.x;
-        unsigned v = i < nb ? bsum[i] : 0u;
-        unsigned tot;
-        unsigned ex = block_excl_scan(v, sm, tot);
-        if (i < nb) bsum[i] = carry + ex;
-        carry += tot;
-    }
-    if (threadIdx.x == 0) bsum[nb] = carry;
-}
-
-template <typename In>
-__global__ void k_scan_apply(const In* __restrict__ in, int n, const unsigned* __restrict__ bsum,
-                             unsigned* __restrict__ out) {
-    __shared__ unsigned sm[32];
-    int base = blockIdx.x * kScanTile + threadIdx.x * kScanIPT;
-    unsigned v[kScanIPT], s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanIPT; ++k) {
-        v[k] = (base + k < n) ? (unsigned)in[base + k] : 0u;
-        s += v[k];
-    }
-    unsigned tot;
-    unsigned ex = block_excl_scan(s, sm, tot) + bsum[blockIdx.x];
-#pragma unroll
-    for (int k = 0; k < kScanIPT; ++k) {
-        if (base + k < n) out[base + k] = ex;
-        ex += v[k];
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = bsum[gridDim.x];
-}
-
-template <typename In>
-void scan_exclusive(const In* in, int n, uint32_t* out, uint32_t* tmp, cudaStream_t s, unsigned* nl) {
-    int nb = (n + kScanTile - 1) / kScanTile;
-    if (nb == 0) {
-        cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
-        return;
-    }
-    k_scan_reduce<In><<<nb, kScanT, 0, s>>>(in, n, tmp);
-    k_scan_bsums<<<1, 1024, 0, s>>>(tmp, nb);
-    k_scan_apply<In><<<nb, kScanT, 0, s>>>(in, n, tmp, out);
-    *nl += 3;
-}
-template void scan_exclusive<uint8_t>(const uint8_t*, int, uint32_t*, uint32_t*, cudaStream_t, unsigned*);
-
-// ---------------------------------------------------------------------------
 // a2: stable LSD radix sort of (64-bit key, 32-bit index), 9-bit digits
 // ---------------------------------------------------------------------------
 //
@@ -582,8 +485,7 @@ __global__ void __launch_bounds__(kTreeTopT) k_hmax_top(const BoxDesc* __restric
 // a6: active list
 // ---------------------------------------------------------------------------
 
-// all particles active: the identity list, and its length where the subset
-// path leaves the compacted count (scan[n])
+// all particles active: the identity list, and its length
 __global__ void k_iota_count(int32_t* a, int n, uint32_t* count) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) a[k] = k;
@@ -600,10 +502,89 @@ __global__ void k_mark(const int32_t* __restrict__ active, int na, const int32_t
     flag[rank[i]] = 1;
 }
 
-__global__ void k_compact(const uint8_t* __restrict__ flag, const uint32_t* __restrict__ scan, int n,
-                          int32_t* __restrict__ act) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n && flag[k]) act[scan[k]] = k;
+// The indices whose flag is set, ascending, and their number, in one pass:
+// a tile of 4096 flags counts its own, publishes the count, and adds the counts
+// of the tiles before it (as k_rs_pass; 32 of them at a time). flag: a byte per
+// index, or (max_bin >= 0) its time bin, set if the bin ends a step at `tick`.
+// work: a ticket and a word per tile, cleared. One launch in place of a
+// three-launch scan and a placing pass over every flag and its scan.
+constexpr int kCpT = 256, kCpPer = 16;
+static_assert(kCpTile == kCpT * kCpPer, "flags per block");
+__global__ void __launch_bounds__(kCpT) k_flag_list(const uint8_t* __restrict__ flag, int n, long long tick, int max_bin,
+                                                    unsigned long long* work, int32_t* __restrict__ list,
+                                                    uint32_t* __restrict__ count, Counters* ctr) {
+    __shared__ unsigned s_tile, s_before, s_warp[kCpT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_tile = atomicAdd(reinterpret_cast<unsigned*>(work), 1u);
+    __syncthreads();
+    const int tile = (int)s_tile;
+    unsigned long long* status = work + 1;
+    const long long i0 = (long long)tile * kCpTile + tid * kCpPer;
+    unsigned set = 0u;   // bit k: flag i0 + k
+    auto take = [&](int k, unsigned v) {
+        if (max_bin >= 0) {
+            const int b = min((int)v, max_bin);
+            v = (tick & ((1ll << (max_bin - b)) - 1)) == 0 ? 1u : 0u;
+        }
+        set |= v ? 1u << k : 0u;
+    };
+    if (i0 + kCpPer <= n && (reinterpret_cast<uintptr_t>(flag) & 15) == 0) {
+        const uint4 v = *reinterpret_cast<const uint4*>(flag + i0);
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < kCpPer; ++k) take(k, (w[k >> 2] >> (8 * (k & 3))) & 255u);
+    } else {
+        for (int k = 0; k < kCpPer; ++k)
+            if (i0 + k < n) take(k, flag[i0 + k]);
+    }
+    const unsigned c = __popc(set);
+    unsigned x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    unsigned before = x - c, total = 0u;
+#pragma unroll
+    for (int w = 0; w < kCpT / 32; ++w) {
+        before += w < warp ? s_warp[w] : 0u;
+        total += s_warp[w];
+    }
+    if (warp == 0) {
+        constexpr unsigned kAgg = 1u, kIncl = 2u;
+        if (lane == 0) rs_put(status + tile, tile == 0 ? kIncl : kAgg, total);
+        unsigned prefix = 0u;
+        int t = tile - 1;
+        for (int spins = 0; t >= 0;) {
+            const unsigned long long w = t >= lane ? rs_get(status + (t - lane)) : (unsigned long long)kIncl << 32;
+            const unsigned tag = (unsigned)(w >> 32);
+            const unsigned incl = __ballot_sync(0xffffffffu, tag == kIncl);
+            const unsigned wait = __ballot_sync(0xffffffffu, tag != kIncl && tag != kAgg);
+            const int fi = incl ? __ffs(incl) - 1 : 32, fw = wait ? __ffs(wait) - 1 : 32;
+            const int use = fi < fw ? fi + 1 : fw;   // words that count: up to the first running total
+            prefix += warp_sum(lane < use ? (unsigned)w : 0u);
+            t = fi < fw ? -1 : t - fw;
+            if (fw < fi && ++spins > kRsSpin) {
+                if (lane == 0 && ctr) atomicOr(&ctr->status, ST_TIMEOUT);
+                break;
+            }
+        }
+        if (lane == 0) {
+            if (tile > 0 && t < 0) rs_put(status + tile, kIncl, prefix + total);
+            s_before = prefix;
+            if ((long long)(tile + 1) * kCpTile >= n) *count = min(prefix + total, (unsigned)n);
+        }
+    }
+    __syncthreads();
+    unsigned pos = s_before + before;
+    while (set) {
+        const int k = __ffs(set) - 1;
+        set &= set - 1u;
+        if (pos < (unsigned)n) list[pos] = (int32_t)(i0 + k);
+        ++pos;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -623,7 +604,7 @@ __global__ void k_compact(const uint8_t* __restrict__ flag, const uint32_t* __re
 void grid_free(sph_grid* g) {
     if (!g) return;
     void* ptrs[] = {g->boxes, g->posm, g->xq, g->perm, g->rank, g->keys, g->node_lo, g->node_hi,
-                    g->node_hmax, g->act, g->flag, g->scan, g->scan_tmp, g->list_a, g->list_b, g->st_lo, g->st_hi, g->list_n, g->d_off, g->d_L,
+                    g->node_hmax, g->act, g->flag, g->act_n, g->list_a, g->list_b, g->st_lo, g->st_hi, g->list_n, g->d_off, g->d_L,
                     g->k2, g->v2, g->rs_work, g->node_c, g->node_e, g->posf,
                     g->fvel, g->fthermo, g->fposh, g->fvm, g->fbal, g->fcond, g->fvisc, g->node_m, g->grav_box, g->nbr, g->nbr_off, g->nbr_n, g->ext_n, g->ext, g->list_xh, g->list_st, g->fb_list, g->list_ep, g->mp_x, g->bw_ga, g->bw_xbar, g->bw_rd, g->bw_f, g->mp_j, g->den_left};
     for (void* p : ptrs)
@@ -707,7 +688,6 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
     g->max_leaves = maxleaf;
     g->max_lev = maxlev;
 
-    const int tmp_words = n / kScanTile + 4;
     GRID_CHECK(cudaMalloc(&g->boxes, sizeof(BoxDesc) * nb));
     GRID_CHECK(cudaMemcpyAsync(g->boxes, g->boxes_h.data(), sizeof(BoxDesc) * nb, cudaMemcpyHostToDevice, s));
     GRID_CHECK(cudaMalloc(&g->d_off, sizeof(long long) * (nb + 1)));
@@ -770,9 +750,9 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
         }
     }
     GRID_CHECK(cudaMalloc(&g->act, sizeof(int32_t) * n));
-    GRID_CHECK(cudaMalloc(&g->flag, n));
-    GRID_CHECK(cudaMalloc(&g->scan, sizeof(uint32_t) * (n + 1)));
-    GRID_CHECK(cudaMalloc(&g->scan_tmp, sizeof(uint32_t) * tmp_words));
+    GRID_CHECK(cudaMemsetAsync(g->act, 0, sizeof(int32_t) * n, s));
+    GRID_CHECK(cudaMalloc(&g->flag, flag_bytes(n) + flag_work_bytes(n)));
+    GRID_CHECK(cudaMalloc(&g->act_n, sizeof(uint32_t)));
     GRID_CHECK(cudaMalloc(&g->list_a, sizeof(int32_t) * n));
     GRID_CHECK(cudaMalloc(&g->list_b, sizeof(int32_t) * n));
     GRID_CHECK(cudaMalloc(&g->st_lo, sizeof(float) * n));
@@ -808,22 +788,29 @@ void grid_refresh_hmax(sph_grid* g, const float* h, cudaStream_t s) {
     }
 }
 
+void flag_list(sph_grid* g, const uint8_t* flag, long long tick, int max_bin, int32_t* list, uint32_t* count,
+               cudaStream_t s) {
+    const int n = (int)g->n;
+    k_flag_list<<<(n + kCpTile - 1) / kCpTile, kCpT, 0, s>>>(flag, n, tick, max_bin,
+                                                             (unsigned long long*)(g->flag + flag_bytes(n)), list, count,
+                                                             g->ctx->counters);
+    ++g->ctx->launches;
+}
+
 void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStream_t s) {
     int n = (int)g->n;
     unsigned& nl = g->ctx->launches;
     if (!active) {
-        k_iota_count<<<(n + 255) / 256, 256, 0, s>>>(g->act, n, g->scan + n);
+        k_iota_count<<<(n + 255) / 256, 256, 0, s>>>(g->act, n, g->act_n);
         ++nl;
     } else {
-        cudaMemsetAsync(g->flag, 0, n, s);
+        cudaMemsetAsync(g->flag, 0, flag_bytes(n) + flag_work_bytes(n), s);   // flags and flag_list's words
         if (n_active > 0) {
             k_mark<<<(int)((n_active + 255) / 256), 256, 0, s>>>(active, (int)n_active, g->rank, g->flag, n,
                                                                   g->ctx->counters);
             ++nl;
         }
-        scan_exclusive<uint8_t>(g->flag, n, g->scan, g->scan_tmp, s, &nl);
-        k_compact<<<(n + 255) / 256, 256, 0, s>>>(g->flag, g->scan, n, g->act);
-        ++nl;
+        flag_list(g, g->flag, 0, -1, g->act, g->act_n, s);
     }
 }
 

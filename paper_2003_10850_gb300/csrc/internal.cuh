@@ -57,9 +57,8 @@ struct sph_grid {
     unsigned char* grav_box = nullptr;     // per gravity call, per box: the cutoff (kGravBoxBytes each)
     // per-call scratch, sized at build so that calls never allocate
     int32_t* act = nullptr;                // active particles, sorted indices, sorted order
-    uint8_t* flag = nullptr;               // n
-    uint32_t* scan = nullptr;              // n + 1
-    uint32_t* scan_tmp = nullptr;          // block sums
+    uint8_t* flag = nullptr;               // flag_bytes(n) flags, then flag_list's words
+    uint32_t* act_n = nullptr;             // length of act
     // plain-path scratch
     int32_t* list_a = nullptr;
     int32_t* list_b = nullptr;
@@ -133,11 +132,15 @@ static_assert(kTreeT % (kFan * kFan) == 0, "whole level-2 nodes per block");
 sph_status grid_update(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s);
 // hmax of every node from the caller-order h
 void grid_refresh_hmax(sph_grid* g, const float* h, cudaStream_t s);
-// active list: sorted indices in g->act, count in g->scan[n]
+// active list: sorted indices in g->act, count in *g->act_n
 void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStream_t s);
-// exclusive scan of n values into out[0..n] (out[n] = total); tmp >= n/4096+2 words
-template <typename In>
-void scan_exclusive(const In* in, int n, uint32_t* out, uint32_t* tmp, cudaStream_t s, unsigned* launches);
+// The set flags' indices, ascending, in list and their number in *count. The words
+// behind g->flag must be clear; flag as k_flag_list in grid.cu.
+constexpr int kCpTile = 4096;
+constexpr size_t flag_bytes(int64_t n) { return ((size_t)n + 15) / 16 * 16; }
+constexpr size_t flag_work_bytes(int64_t n) { return 8 * ((size_t)(n + kCpTile - 1) / kCpTile + 1); }
+void flag_list(sph_grid* g, const uint8_t* flag, long long tick, int max_bin, int32_t* list, uint32_t* count,
+               cudaStream_t s);
 // stable radix sort of (key, index) pairs, see grid.cu; work: rs_work_bytes(n) bytes, 16-byte aligned
 constexpr int kRsBits = 9;          // bits per pass
 constexpr int kRsTile = 4096;       // items per block

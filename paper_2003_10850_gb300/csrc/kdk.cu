@@ -43,27 +43,6 @@ __global__ void k_timebins(int n, const float* __restrict__ h, const float* __re
     bins[i] = (uint8_t)b;
 }
 
-__global__ void k_active_flags(int n, const uint8_t* __restrict__ bins, long long tick, int max_bin,
-                               uint8_t* __restrict__ flag) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int b = min((int)bins[i], max_bin);
-    flag[i] = (tick & ((1ll << (max_bin - b)) - 1)) == 0 ? 1 : 0;
-}
-
-// The active particles ascending in active[0, count), then -1 in every entry
-// of active[count, n): the whole array can be passed on with n_active = n,
-// without reading the count on the host (negative entries are skipped).
-__global__ void k_flags_to_list(int n, const uint8_t* __restrict__ flag, const uint32_t* __restrict__ scan,
-                                int32_t* __restrict__ active, int32_t* __restrict__ count) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        if (flag[i]) active[scan[i]] = i;
-        else active[scan[n] + (i - scan[i])] = -1;
-    }
-    if (i == 0) *count = (int32_t)scan[n];
-}
-
 struct KickSteps {
     float dt[32];
 };
@@ -183,10 +162,10 @@ sph_status sph_active_from_bins(sph_ctx* ctx, sph_grid* grid, const uint8_t* bin
     if (cudaSetDevice(ctx->device)) return kdk_fail(ctx, SPH_ERR_CUDA, "cudaSetDevice failed");
     cudaStream_t s = (cudaStream_t)stream;
     const int n = (int)grid->n;
-    k_active_flags<<<(n + 255) / 256, 256, 0, s>>>(n, bins, (long long)tick, max_bin, grid->flag);
-    scan_exclusive<uint8_t>(grid->flag, n, grid->scan, grid->scan_tmp, s, &ctx->launches);
-    k_flags_to_list<<<(n + 255) / 256, 256, 0, s>>>(n, grid->flag, grid->scan, active, n_active);
-    ctx->launches += 2;
+    // ascending in active[0, count), -1 in every entry past it
+    cudaMemsetAsync(active, 0xff, sizeof(int32_t) * (size_t)n, s);
+    cudaMemsetAsync(grid->flag + flag_bytes(n), 0, flag_work_bytes(n), s);
+    flag_list(grid, bins, (long long)tick, max_bin, active, reinterpret_cast<uint32_t*>(n_active), s);
     return cudaGetLastError() ? kdk_fail(ctx, SPH_ERR_CUDA, "sph_active_from_bins launch failed") : SPH_OK;
 }
 

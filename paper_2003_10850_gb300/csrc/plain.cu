@@ -321,7 +321,7 @@ cudaError_t run_density_plain(sph_ctx* ctx, const DensityLaunch& a, int64_t n_ac
     // the first pass reads the active count from the device (the compacted
     // active list drops duplicates); later passes read it back to decide
     int count = (int)n_active;
-    const int* count0 = reinterpret_cast<const int*>(g->scan + g->n);
+    const int* count0 = reinterpret_cast<const int*>(g->act_n);
     const int32_t* list = g->act;
     int32_t* bufs[2] = {g->list_a, g->list_b};
     int which = 0;
@@ -355,7 +355,7 @@ cudaError_t launch_force_plain(sph_ctx* ctx, const ForceLaunch& a, int64_t n_act
     pa.n_boxes = g->n_boxes;
     pa.act = g->act;
     pa.count = (int)n_active;
-    pa.count_ptr = reinterpret_cast<const int*>(g->scan + g->n);
+    pa.count_ptr = reinterpret_cast<const int*>(g->act_n);
     pa.posm = g->posm;
     pa.perm = g->perm;
     pa.node_lo = g->node_lo;

@@ -691,7 +691,7 @@ cudaError_t launch_density_tpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
     da.boxes = g->boxes;
     da.n_boxes = g->n_boxes;
     da.act = g->act;
-    da.count_ptr = reinterpret_cast<const int*>(g->scan + g->n);
+    da.count_ptr = reinterpret_cast<const int*>(g->act_n);
     da.count = (int)n_active;
     da.posm = g->posm;
     da.posf = g->posf;
@@ -738,7 +738,7 @@ cudaError_t launch_force_tpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_activ
     fa.boxes = g->boxes;
     fa.n_boxes = g->n_boxes;
     fa.act = g->act;
-    fa.count_ptr = reinterpret_cast<const int*>(g->scan + g->n);
+    fa.count_ptr = reinterpret_cast<const int*>(g->act_n);
     fa.count = (int)n_active;
     fa.posm = g->posm;
     fa.posf = g->posf;

@@ -756,7 +756,7 @@ static inline WppArgs wpp_common(sph_ctx* ctx, const sph_grid* g, unsigned* queu
     c.boxes = g->boxes;
     c.n_boxes = g->n_boxes;
     c.act = g->act;
-    c.count_ptr = g->scan + g->n;
+    c.count_ptr = g->act_n;
     c.queue = queue;
     c.posm = g->posm;
     c.posf = g->posf;

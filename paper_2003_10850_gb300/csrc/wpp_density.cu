@@ -1333,7 +1333,7 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
     if (rec) {
         const int n = (int)g->n, hb = helper_blocks(ctx, n);
         const int32_t* act = part ? g->act : nullptr;
-        const uint32_t* count = g->scan + n;
+        const uint32_t* count = g->act_n;
         k_list_ext<<<hb, 256, 0, s>>>(g->boxes, g->n_boxes, n, g->posm, g->nbr, g->nbr_off, g->nbr_n, g->list_xh,
                                       g->ext_n, g->ext, g->list_st, act, count, g->flag, g->list_ep);
         k_list_sort<<<hb, 256, 0, s>>>(n, g->ext, g->ext_n, g->list_st, act, count);
