@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
     c_lists = warp_sum(c_lists);
     c_tests = warp_sum(c_tests);
     c_status = __reduce_or_sync(0xffffffffu, c_status);
-    if (lane == 0) {
+    if (lane == 0 && c_tests) {
         if (a.nbr && c_lists) atomicAdd(&a.list_st[0], c_lists);
         atomicAdd(&a.ctr->density_pairs, (unsigned long long)c_pairs);
         atomicAdd(&a.ctr->density_evals, (unsigned long long)c_evals);
@@ -594,6 +594,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
     const float rel = 9.5367431640625e-07f;  // 2^-20
     const float nt = (float)a.n_target, nt3 = 3.f * nt, tol3 = 3.f * (float)a.n_tol;
     const int cnt = (int)*a.count_ptr;
+    if (cnt == 0) return;   // (before thousands of warps queue for nothing)
     unsigned c_pairs = 0, c_evals = 0, c_tests = 0, c_status = 0, c_lists = 0;   // per warp (32-bit suffices)
     long long ch_next = 0, ch_end = 0;   // the warp's current chunk of the neighbour-list pool
     for (;;) {
@@ -975,7 +976,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
         }
     }
     const unsigned long long all_tests = c_tests;   // counted warp-uniformly
-    if (lane == 0) {
+    if (lane == 0 && c_evals) {
         if (a.nbr && c_lists) atomicAdd(&a.list_st[0], c_lists);
         atomicAdd(&a.ctr->density_pairs, (unsigned long long)c_pairs);
         atomicAdd(&a.ctr->density_evals, (unsigned long long)c_evals);
@@ -1104,10 +1105,11 @@ __global__ void __launch_bounds__(256) k_list_ext(const BoxDesc* __restrict__ bo
 // force pass's sums): up to 64 entries each goes to its rank (registers), up
 // to kExtCap through a bitonic sort in shared memory. A segment that
 // overflowed is marked kExtUnusable, and the force pass walks for that
-// particle. A warp reads the counts of 32 particles at a time and sorts their
-// segments one after another.
-__global__ void __launch_bounds__(256) k_list_sort(int n, int32_t* __restrict__ ext, uint32_t* __restrict__ ext_n,
-                                                   const unsigned* __restrict__ list_st,
+// particle. A warp reads the counts of `per` particles at a time (few, so that
+// small sets spread over all warps) and sorts their segments one after another,
+// the next one's entries loaded while this one is sorted.
+__global__ void __launch_bounds__(256) k_list_sort(int n, int per, int32_t* __restrict__ ext,
+                                                   uint32_t* __restrict__ ext_n, const unsigned* __restrict__ list_st,
                                                    const int32_t* __restrict__ act, const uint32_t* __restrict__ count) {
     if (list_st[1] != 0u) return;   // the lists cannot serve a force call
     __shared__ int buf[8][kExtCap];
@@ -1115,45 +1117,59 @@ __global__ void __launch_bounds__(256) k_list_sort(int n, int32_t* __restrict__ 
     const unsigned lane = lane_id();
     const int warps = gridDim.x * (blockDim.x >> 5);
     const int ni = act ? (int)*count : n;
-    for (int t0 = (blockIdx.x * (blockDim.x >> 5) + (int)(threadIdx.x >> 5)) * 32; t0 < ni; t0 += warps * 32) {
+    int iln = -1;
+    unsigned cln = 0u;
+    auto counts = [&](int t0) {
         const int tl = t0 + (int)lane;
-        const int il = tl < ni ? (act ? act[tl] : tl) : -1;
-        const unsigned cl = il >= 0 ? ext_n[il] : 0u;
+        iln = (int)lane < per && tl < ni ? (act ? act[tl] : tl) : -1;
+        cln = iln >= 0 ? ext_n[iln] : 0u;
+    };
+    int t0 = (blockIdx.x * (blockDim.x >> 5) + (int)(threadIdx.x >> 5)) * per;
+    counts(t0);
+    for (; t0 < ni; t0 += warps * per) {
+        const int il = iln;
+        const unsigned cl = cln;
+        counts(t0 + warps * per);
         if (cl > (unsigned)kExtCap) ext_n[il] = kExtUnusable;
         unsigned todo = __ballot_sync(0xffffffffu, cl >= 2u && cl <= (unsigned)kExtCap);
-        while (todo) {
+        int i = 0, c = 0, v0 = 0, v1 = 0;
+        auto fetch = [&]() {   // the next segment: its first 64 entries, two per lane
             const int src = __ffs(todo) - 1;
             todo &= todo - 1u;
-            const int i = __shfl_sync(0xffffffffu, il, src);
-            const int c = (int)__shfl_sync(0xffffffffu, cl, src);
+            i = __shfl_sync(0xffffffffu, il, src);
+            c = (int)__shfl_sync(0xffffffffu, cl, src);
+            const int32_t* seg = ext + (size_t)i * kExtCap;
+            v0 = (int)lane < c ? seg[lane] : 0x7fffffff;
+            v1 = (int)lane + 32 < c ? seg[lane + 32] : 0x7fffffff;
+        };
+        bool more = todo != 0u;
+        if (more) fetch();
+        while (more) {
+            const int cc = c, w0 = v0, w1 = v1;
             int32_t* seg = ext + (size_t)i * kExtCap;
-            if (c <= 32) {   // one entry per lane: its rank among the c
-                const int v0 = (int)lane < c ? seg[lane] : 0x7fffffff;
-                int r0 = 0;
-                for (int k = 0; k < c; ++k) r0 += __shfl_sync(0xffffffffu, v0, k) < v0;
-                __syncwarp();   // every lane has read the segment before it is overwritten
-                if ((int)lane < c) seg[r0] = v0;
-            } else if (c <= 64) {
-                const int v0 = (int)lane < c ? seg[lane] : 0x7fffffff;
-                const int v1 = (int)lane + 32 < c ? seg[lane + 32] : 0x7fffffff;
+            more = todo != 0u;
+            if (more) fetch();
+            if (cc <= 64) {   // one or two entries per lane: the rank among the cc
                 int r0 = 0, r1 = 0;
-                const int c0 = min(c, 32);
+                const int c0 = min(cc, 32);
                 for (int k = 0; k < c0; ++k) {
-                    const int x = __shfl_sync(0xffffffffu, v0, k);
-                    r0 += x < v0;
-                    r1 += x < v1;
+                    const int x = __shfl_sync(0xffffffffu, w0, k);
+                    r0 += x < w0;
+                    r1 += x < w1;
                 }
-                for (int k = 32; k < c; ++k) {
-                    const int x = __shfl_sync(0xffffffffu, v1, k - 32);
-                    r0 += x < v0;
-                    r1 += x < v1;
+                for (int k = 32; k < cc; ++k) {
+                    const int x = __shfl_sync(0xffffffffu, w1, k - 32);
+                    r0 += x < w0;
+                    r1 += x < w1;
                 }
                 __syncwarp();   // every lane has read the segment before it is overwritten
-                if ((int)lane < c) seg[r0] = v0;
-                if ((int)lane + 32 < c) seg[r1] = v1;
+                if ((int)lane < cc) seg[r0] = w0;
+                if ((int)lane + 32 < cc) seg[r1] = w1;
             } else {
                 constexpr int P = kExtCap;   // a power of two
-                for (int k = (int)lane; k < P; k += 32) sb[k] = k < c ? seg[k] : 0x7fffffff;
+                sb[lane] = w0;
+                sb[lane + 32] = w1;
+                for (int k = (int)lane + 64; k < P; k += 32) sb[k] = k < cc ? seg[k] : 0x7fffffff;
                 __syncwarp();
                 for (int size = 2; size <= P; size <<= 1) {
                     for (int stride = size >> 1; stride > 0; stride >>= 1) {
@@ -1169,9 +1185,9 @@ __global__ void __launch_bounds__(256) k_list_sort(int n, int32_t* __restrict__ 
                         __syncwarp();
                     }
                 }
-                for (int k = (int)lane; k < c; k += 32) seg[k] = sb[k];
+                for (int k = (int)lane; k < cc; k += 32) seg[k] = sb[k];
+                __syncwarp();
             }
-            __syncwarp();
         }
     }
 }
@@ -1336,7 +1352,8 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
         const uint32_t* count = g->act_n;
         k_list_ext<<<hb, 256, 0, s>>>(g->boxes, g->n_boxes, n, g->posm, g->nbr, g->nbr_off, g->nbr_n, g->list_xh,
                                       g->ext_n, g->ext, g->list_st, act, count, g->flag, g->list_ep);
-        k_list_sort<<<hb, 256, 0, s>>>(n, g->ext, g->ext_n, g->list_st, act, count);
+        const int per = (int)std::min<long long>(8, ((long long)n + 8ll * hb - 1) / (8ll * hb));
+        k_list_sort<<<hb, 256, 0, s>>>(n, per, g->ext, g->ext_n, g->list_st, act, count);
         ctx->launches += 2;
     }
     g->lists_rec = rec;

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_wpp(WppArgs a) {
         cnt = (int)*a.left_n;
         chunk = 1;
     }
+    if (cnt == 0) return;   // (before thousands of warps queue for nothing)
     unsigned long long c_pairs = 0, c_tests = 0;   // lane 0's per-warp totals
     for (;;) {
         int t0 = 0;
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_wpp(WppArgs a) {
             }
         }
     }
-    if (lane == 0) {
+    if (lane == 0 && c_tests) {
         atomicAdd(&a.ctr->force_pairs, c_pairs);
         atomicAdd(&a.ctr->pair_tests, c_tests);
     }
@@ -628,7 +629,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
             }
         }
     }
-    if (lane == 0) {
+    if (lane == 0 && c_tests) {
         atomicAdd(&a.ctr->force_pairs, c_pairs);
         atomicAdd(&a.ctr->pair_tests, c_tests);
     }
