@@ -153,6 +153,9 @@ struct WppArgs {
     // density: the particles the member-parallel kernel leaves to the one-particle kernel
     int32_t* left;
     unsigned* left_n;
+    // force: the member-parallel kernel's rule on the device's own active count
+    // (wpp_groups_pay; 0: none); when it fails the one-particle kernel takes the whole set
+    int mp_min;
     // lists of a partial active set: the active flag per sorted particle, the
     // far-partner scratch (kMpMembers x kMpFar per warp), and the generation
     // stamp per particle (a list serves only if its stamp is the current one)
@@ -166,6 +169,12 @@ struct WppArgs {
 // particle's own list is from the last density call is its list_ep stamp.)
 __device__ __forceinline__ bool wpp_lists_valid(const unsigned* st) {
     return st[1] == 0u && st[2] == 0u;
+}
+
+// The rule of wpp_groups_pay for the count a kernel finds: a list padded to its
+// capacity (a time-stepping loop's) tells the host nothing about its length.
+__device__ __forceinline__ bool wpp_count_pays(int cnt, int mp_min, int n_total) {
+    return mp_min == 0 || (cnt >= mp_min && (long long)cnt * 256 >= n_total);
 }
 
 __device__ __forceinline__ int wpp_box(const BoxDesc* boxes, int nb, long long p) {
@@ -777,8 +786,9 @@ static inline WppArgs wpp_common(sph_ctx* ctx, const sph_grid* g, unsigned* queu
 // particles are not too sparse to share leaves (at least 1 in 256 active).
 // Measured on 10M clustered particles with time-bin active sets: 1% active
 // (100k) runs faster in groups, 0.1% (10k) slower.
-static inline bool wpp_groups_pay(const sph_ctx* ctx, int64_t n_active, int64_t n) {
-    return n_active >= (int64_t)kMpMembers * 16 * ctx->sm_count && n_active * 256 >= n;
+static inline int wpp_mp_min(const sph_ctx* ctx, int warps) { return kMpMembers * warps * ctx->sm_count; }
+static inline bool wpp_groups_pay(const sph_ctx* ctx, int64_t n_active, int64_t n, int warps = 16) {
+    return n_active >= wpp_mp_min(ctx, warps) && n_active * 256 >= n;
 }
 
 // Grid of a warp-per-particle helper kernel over n particles (256 threads).

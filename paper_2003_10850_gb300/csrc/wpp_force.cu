@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_wpp(WppArgs a) {
         act = a.fb_act;
         cnt = (int)*a.fb_count;
         chunk = 1;
-    } else if (a.left) {   // after the member-parallel walk: the particles it left
+    } else if (a.left && wpp_count_pays(cnt, a.mp_min, a.n_total)) {   // after the member-parallel walk: what it left
         act = a.left;
         cnt = (int)*a.left_n;
         chunk = 1;
@@ -327,6 +327,12 @@ __global__ void __launch_bounds__(128, 8) k_force_list(WppArgs a) {
 // whose leaf list overflows and members whose pair list overflows are left
 // to the one-particle walk (k_force_wpp).
 constexpr int kFmCap = 256;   // pairs per member in the scratch list
+// The groups must fill the GPU several times over (warps' worth of full groups
+// per SM): one group takes about 0.2 ms. Clustered sets, us walked in groups / one
+// particle per warp: 24,000 of 200,000 308 / 226, 20,971 of 2M 439 / 278, 40,000 of
+// 4M 547 / 458, 62,914 of 2M 528 / 547, 100,000 of 200,000 540 / 622, 209,715 of 2M
+// 1028 / 1467.
+constexpr int kFmMinWarps = 48;
 static_assert(kMpMembers * kFmCap <= 2 * kMpMembers * kMpCap, "scratch of a force warp");
 
 struct WppFmSmem {
@@ -348,6 +354,7 @@ template <bool HASH, int MINB, int VISC, bool COND>
 __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
     // the recorded lists served this call: the walk takes only their fallbacks
     if (a.fb_act && wpp_lists_valid(a.list_st)) return;
+    if (!wpp_count_pays((int)*a.count_ptr, a.mp_min, a.n_total)) return;
     __shared__ WppFmSmem smem[kWppWarps];
     const int wib = (int)(threadIdx.x >> 5);
     WppFmSmem& sm = smem[wib];
@@ -733,9 +740,10 @@ cudaError_t launch_force_wpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_activ
     // the walk: member-parallel for groups (nothing to do when the lists served
     // the call), then one particle per warp for what it leaves and for the
     // particles the lists could not serve
-    if (g->ctx->sm_count >= ctx->sm_count && wpp_groups_pay(ctx, n_active, g->n)) {
+    if (g->ctx->sm_count >= ctx->sm_count && wpp_groups_pay(ctx, n_active, g->n, kFmMinWarps)) {
         if ((e = cudaMemsetAsync(ctx->queue + 6, 0, 2 * sizeof(unsigned), s))) return e;
         WppArgs cm = c;
+        c.mp_min = cm.mp_min = wpp_mp_min(ctx, kFmMinWarps);
         cm.mp_j = g->mp_j;
         cm.left = g->den_left;
         cm.left_n = ctx->queue + 6;
