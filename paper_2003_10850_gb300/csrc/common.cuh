@@ -170,6 +170,16 @@ __device__ __forceinline__ void spline(T q, T& w, T& dw) {
     dw = T(24) * b2 - T(6) * a2;
 }
 
+// w'(q) for two arguments at once.
+__device__ __forceinline__ float2 spline_dw2(float2 q) {
+    float2 a = sub2(both(1.f), q), b = sub2(both(0.5f), q);
+    a.x = fmaxf(a.x, 0.f);
+    a.y = fmaxf(a.y, 0.f);
+    b.x = fmaxf(b.x, 0.f);
+    b.y = fmaxf(b.y, 0.f);
+    return fma2(mul2(both(24.f), b), b, mul2(mul2(both(-6.f), a), a));
+}
+
 // Compensated (Kahan) addition of x into (s, c); explicit round-to-nearest
 // intrinsics keep the compensation from being reassociated or contracted.
 __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {

@@ -714,6 +714,60 @@ __device__ __forceinline__ void wpp_force_pair(const WppForceI& I, float dx, flo
     Su += mj * vr * (I.A * Fi + 0.5f * PI * Fbar);
 }
 
+// Per-lane sums of the list passes, two pairs at a time.
+struct WppForceS2 {
+    float2 x = {0.f, 0.f}, y = {0.f, 0.f}, z = {0.f, 0.f}, u = {0.f, 0.f}, c = {0.f, 0.f};   // u: -du/dt
+    float vsmax = 0.f;
+};
+
+// The terms of two pairs in packed arithmetic: half the FP32 instructions, the
+// largest part of what the list passes issue between their gathers. d = x_j - x_i, v = (v_j, m_j), th =
+// (rho_j, A_j, c_j, 1/h_j), b and c as wpp_force_pair; two false: the second
+// pair is none. A coincident pair adds its sound speeds to v_sig and no force.
+template <int VISC, bool COND>
+__device__ __forceinline__ void wpp_force_pair2(const WppForceI& I, float2 dx, float2 dy, float2 dz, float4 v0, float4 v1,
+                                                float4 th0, float4 th1, float2 b0, float2 b1, float2 c0, float2 c1,
+                                                float alpha, bool two, WppForceS2& S) {
+    float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+    float2 m = make_float2(v0.w, two ? v1.w : 0.f);
+    if (r2.x <= 0.f) { r2.x = 1.f; m.x = 0.f; }
+    if (r2.y <= 0.f) { r2.y = 1.f; m.y = 0.f; }
+    const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y)), r = mul2(r2, rinv);
+    const float2 hj = make_float2(th0.w, th1.w), hj2 = mul2(hj, hj);
+    const float2 Fi = mul2(mul2(both(I.norm), spline_dw2(mul2(r, both(I.hinv)))), rinv);
+    const float2 Fj = mul2(mul2(mul2(both((float)(8.0 / 3.141592653589793)), mul2(hj2, hj2)), spline_dw2(mul2(r, hj))),
+                           rinv);
+    // t = -v_ij . r_ij (r_ij = -d), w = -w_ij
+    const float2 t = fma2(sub2(both(I.vz), make_float2(v0.z, v1.z)), dz,
+                          fma2(sub2(both(I.vy), make_float2(v0.y, v1.y)), dy,
+                               mul2(sub2(both(I.vx), make_float2(v0.x, v1.x)), dx)));
+    const float2 w = mul2(t, rinv);
+    const float2 vs = fma2(both(3.f), w, add2(both(I.c), make_float2(th0.z, th1.z)));
+    S.vsmax = fmaxf(S.vsmax, fmaxf(vs.x, two ? vs.y : 0.f));
+    // Pi_ij = -(alpha/2) v_sig w_ij / rho_bar for w_ij < 0, rho_bar = (rho_i + rho_j)/2
+    const float2 rj = make_float2(th0.x, th1.x);
+    const float2 al = VISC == kViscPerParticle ? mul2(both(0.5f), add2(both(I.al), make_float2(b0.y, b1.y)))
+                                               : both(alpha);
+    const float2 wp = make_float2(fmaxf(w.x, 0.f), fmaxf(w.y, 0.f));
+    float2 PI = mul2(mul2(mul2(al, vs), wp), rcp2_ftz(add2(both(I.rho), rj)));
+    if (VISC != kViscScalar) PI = mul2(PI, mul2(both(0.5f), add2(both(I.f), make_float2(b0.x, b1.x))));
+    const float2 Fbar = mul2(both(0.5f), add2(Fi, Fj)), AF = mul2(both(I.A), Fi);
+    if (COND) {
+        const float2 kj = make_float2(c0.y, c1.y), ks = add2(both(I.kap), kj);
+        float2 kij = mul2(mul2(both(4.f * I.kap), kj), rcp2_ftz(ks));
+        kij.x = ks.x > 0.f ? kij.x : 0.f;
+        kij.y = ks.y > 0.f ? kij.y : 0.f;
+        const float2 mr = mul2(m, rcp2_ftz(mul2(both(I.rho), rj)));
+        S.c = fma2(mul2(mul2(mr, kij), sub2(both(I.u), make_float2(c0.x, c1.x))), Fbar, S.c);
+    }
+    const float2 PF = mul2(PI, Fbar);
+    const float2 coef = mul2(m, add2(fma2(make_float2(th0.y, th1.y), Fj, AF), PF));
+    S.x = fma2(coef, dx, S.x);
+    S.y = fma2(coef, dy, S.y);
+    S.z = fma2(coef, dz, S.z);
+    S.u = fma2(mul2(m, t), fma2(both(0.5f), PF, AF), S.u);
+}
+
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------

@@ -209,8 +209,12 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_wpp(WppArgs a) {
 // does nothing and the walk that follows takes the whole active set;
 // particles whose own lists did not fit go to fb_list for that walk.
 constexpr int kFlPer = 4;   // particles per warp
+// 80 registers (96 with conduction), so that both pairs' records stay in registers:
+// 10M clustered particles (timebins step) 48.1 / 47.9 / 48.9 ms at 8 / 6 / 5 blocks per
+// SM, conduction of 800k 0.96 / 0.90 / 0.84 ms; one pair at a time at 8 blocks took
+// 0.465 ms for 300k particles, this 0.367 (with the scatter of the results).
 template <bool HASH, int VISC, bool COND>
-__global__ void __launch_bounds__(128, 8) k_force_list(WppArgs a) {
+__global__ void __launch_bounds__(128, COND ? 5 : 6) k_force_list(WppArgs a) {
     if (!wpp_lists_valid(a.list_st)) return;
     const unsigned gen = a.list_st[kListGen];
     const unsigned lane = lane_id();
@@ -246,7 +250,7 @@ __global__ void __launch_bounds__(128, 8) k_force_list(WppArgs a) {
         const float2 bi = wpp_visc_i<VISC>(a, pp);
         const WppForceI I = {vi.x, vi.y, vi.z, thi.w, thi.x, thi.y, thi.z, kNorm * thi.w * thi.w * thi.w * thi.w,
                              bi.x, ci.x, ci.y, bi.y};
-        float Sx = 0.f, Sy = 0.f, Sz = 0.f, Su = 0.f, Sc = 0.f, vsmax = 0.f;
+        WppForceS2 S;
         unsigned long long hs = 0;
         const int tot = live ? cn + (int)ec : 0;
         const int32_t* ln = a.nbr + (live ? a.nbr_off[pp] : 0);
@@ -271,25 +275,26 @@ __global__ void __launch_bounds__(128, 8) k_force_list(WppArgs a) {
                 const float2 b0 = wpp_visc_j<VISC>(a, q0), b1 = wpp_visc_j<VISC>(a, q1);
                 const float2 c0 = COND ? __ldg(a.fcond + q0) : make_float2(0.f, 0.f);
                 const float2 c1 = COND ? __ldg(a.fcond + q1) : make_float2(0.f, 0.f);
-                wpp_force_pair<VISC, COND>(I, (float)(int)(X0.x - Xi.x) * sf, (float)(int)(X0.y - Xi.y) * sf,
-                                          (float)(int)(X0.z - Xi.z) * sf, v0, t0v, b0, c0, a.alpha, Sx, Sy, Sz, Su,
-                                          Sc, vsmax);
-                if (HASH) hs += splitmix64((unsigned long long)a.perm[q0]);
-                if (two) {
-                    wpp_force_pair<VISC, COND>(I, (float)(int)(X1.x - Xi.x) * sf, (float)(int)(X1.y - Xi.y) * sf,
-                                              (float)(int)(X1.z - Xi.z) * sf, v1, t1v, b1, c1, a.alpha, Sx, Sy, Sz,
-                                              Su, Sc, vsmax);
-                    if (HASH) hs += splitmix64((unsigned long long)a.perm[q1]);
+                const float2 s2 = both(sf);
+                wpp_force_pair2<VISC, COND>(
+                    I, mul2(make_float2((float)(int)(X0.x - Xi.x), (float)(int)(X1.x - Xi.x)), s2),
+                    mul2(make_float2((float)(int)(X0.y - Xi.y), (float)(int)(X1.y - Xi.y)), s2),
+                    mul2(make_float2((float)(int)(X0.z - Xi.z), (float)(int)(X1.z - Xi.z)), s2), v0, v1, t0v, t1v, b0, b1,
+                    c0, c1, a.alpha, two, S);
+                if (HASH) {
+                    hs += splitmix64((unsigned long long)a.perm[q0]);
+                    if (two) hs += splitmix64((unsigned long long)a.perm[q1]);
                 }
             }
         }
-        const float fs = wpp_fold4_oct(Sx, Sy, Sz, Su);
+        float vsmax = S.vsmax;
+        const float fs = wpp_fold4_oct(S.x.x + S.x.y, S.y.x + S.y.y, S.z.x + S.z.y, -(S.u.x + S.u.y));
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) {
             vsmax = fmaxf(vsmax, __shfl_xor_sync(0xffffffffu, vsmax, o));
             if (HASH) hs += __shfl_xor_sync(0xffffffffu, hs, o);
         }
-        const float cs = COND ? wpp_fold1_oct(Sc) : 0.f;
+        const float cs = COND ? wpp_fold1_oct(S.c.x + S.c.y) : 0.f;
         if (live) {
             if ((sub & 1) == 0) {
                 const int comp = sub >> 1;
@@ -571,7 +576,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
                     const float2 bi = wpp_visc_i<VISC>(a, p);
                     const WppForceI I = {vi.x, vi.y, vi.z, thi.w, thi.x, thi.y, thi.z,
                                          kNorm * thi.w * thi.w * thi.w * thi.w, bi.x, ci.x, ci.y, bi.y};
-                    float Sx = 0.f, Sy = 0.f, Sz = 0.f, Su = 0.f, Sc = 0.f, vsmax = 0.f;
+                    WppForceS2 S;
                     unsigned long long hs = 0;
                     const int32_t* lst = pj + mq * kFmCap;
                     int q0n = sub < tot ? lst[sub] : 0;
@@ -588,26 +593,26 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
                             const float2 b0 = wpp_visc_j<VISC>(a, q0), b1 = wpp_visc_j<VISC>(a, q1);
                             const float2 c0 = COND ? __ldg(a.fcond + q0) : make_float2(0.f, 0.f);
                             const float2 c1 = COND ? __ldg(a.fcond + q1) : make_float2(0.f, 0.f);
-                            wpp_force_pair<VISC, COND>(I, (float)(int)(X0.x - Xi.x) * sf,
-                                                       (float)(int)(X0.y - Xi.y) * sf, (float)(int)(X0.z - Xi.z) * sf,
-                                                       v0, th0, b0, c0, a.alpha, Sx, Sy, Sz, Su, Sc, vsmax);
-                            if (HASH) hs += splitmix64((unsigned long long)a.perm[q0]);
-                            if (two) {
-                                wpp_force_pair<VISC, COND>(I, (float)(int)(X1.x - Xi.x) * sf,
-                                                           (float)(int)(X1.y - Xi.y) * sf,
-                                                           (float)(int)(X1.z - Xi.z) * sf, v1, th1, b1, c1, a.alpha,
-                                                           Sx, Sy, Sz, Su, Sc, vsmax);
-                                if (HASH) hs += splitmix64((unsigned long long)a.perm[q1]);
+                            const float2 s2 = both(sf);
+                            wpp_force_pair2<VISC, COND>(
+                                I, mul2(make_float2((float)(int)(X0.x - Xi.x), (float)(int)(X1.x - Xi.x)), s2),
+                                mul2(make_float2((float)(int)(X0.y - Xi.y), (float)(int)(X1.y - Xi.y)), s2),
+                                mul2(make_float2((float)(int)(X0.z - Xi.z), (float)(int)(X1.z - Xi.z)), s2), v0, v1, th0,
+                                th1, b0, b1, c0, c1, a.alpha, two, S);
+                            if (HASH) {
+                                hs += splitmix64((unsigned long long)a.perm[q0]);
+                                if (two) hs += splitmix64((unsigned long long)a.perm[q1]);
                             }
                         }
                     }
-                    const float fs = wpp_fold4_oct(Sx, Sy, Sz, Su);
+                    float vsmax = S.vsmax;
+                    const float fs = wpp_fold4_oct(S.x.x + S.x.y, S.y.x + S.y.y, S.z.x + S.z.y, -(S.u.x + S.u.y));
 #pragma unroll
                     for (int o = 4; o > 0; o >>= 1) {
                         vsmax = fmaxf(vsmax, __shfl_xor_sync(0xffffffffu, vsmax, o));
                         if (HASH) hs += __shfl_xor_sync(0xffffffffu, hs, o);
                     }
-                    const float cs = COND ? wpp_fold1_oct(Sc) : 0.f;
+                    const float cs = COND ? wpp_fold1_oct(S.c.x + S.c.y) : 0.f;
                     if (live) {
                         if ((sub & 1) == 0) {
                             const int comp = sub >> 1;
