@@ -170,6 +170,19 @@ __device__ __forceinline__ void spline(T q, T& w, T& dw) {
     dw = T(24) * b2 - T(6) * a2;
 }
 
+// The same for two arguments at once, rounded as the scalar form is compiled
+// (2 a^2 a and 24 b^2 fused with the other product).
+__device__ __forceinline__ void spline_pair(float2 q, float2& w, float2& dw) {
+    float2 a = sub2(both(1.f), q), b = sub2(both(0.5f), q);
+    a.x = fmaxf(a.x, 0.f);
+    a.y = fmaxf(a.y, 0.f);
+    b.x = fmaxf(b.x, 0.f);
+    b.y = fmaxf(b.y, 0.f);
+    const float2 a2 = mul2(a, a), b2 = mul2(b, b);
+    w = fma2(mul2(both(2.f), a2), a, mul2(mul2(both(-8.f), b2), b));
+    dw = fma2(both(24.f), b2, mul2(both(-6.f), a2));
+}
+
 // w'(q) for two arguments at once.
 __device__ __forceinline__ float2 spline_dw2(float2 q) {
     float2 a = sub2(both(1.f), q), b = sub2(both(0.5f), q);

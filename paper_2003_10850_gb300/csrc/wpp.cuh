@@ -49,7 +49,10 @@ constexpr int kWppThreads = kWppWarps * 32;
 // one matching blocks_per_sm; the autotuner picks between them per pass.
 constexpr int kWppDensityBps = 5;
 constexpr int kWppDensityMaxBps = 5;
-constexpr int kWppLeftBps = 6;   // the one-particle density kernel over the leftovers: 80 registers
+// The one-particle density kernel: 5 blocks, 96 registers (6 spill; density call of
+// 262k clustered particles 2.06 / 1.83 / 1.82 ms at 6 / 5 / 4, of 64 boxes 8.4 / 7.7 /
+// 7.7). Its time is the longest particle's: loads run a step ahead of their use.
+constexpr int kWppLeftBps = 5;
 constexpr int kWppFmBps = 6;     // the member-parallel force walk: 80 registers
 constexpr int kWppForceBps = 8;
 constexpr int kWppMaxBps = 16;
@@ -59,6 +62,16 @@ constexpr int kWppPop8 = 96;         // group walk: pop eight nodes per step onl
 constexpr int kWppLeaves = 128;      // leaf list per warp; a step adds <= 32
 constexpr int kWppHits = 64;         // hit buffer per warp; drained at >= 32
 constexpr int kWppNear = 128;        // density: pairs within the walk radius, kept across h iterations
+// A near list of the one-particle density kernel that outgrows kWppNear is kept in
+// the warp's part of the scratch (mp_j, shared by 4 kWppLeftBps warps per SM). A
+// particle beside a compact clump has a few hundred pairs within its walk radius
+// (64 clustered boxes: 1 particle in 13 more than 128, at most 920); sweeping its
+// candidates again for every h iteration took 5 to 15 times the others' time.
+constexpr int kWppFar = 896;
+constexpr int kWppFarBytes = kWppFar * 12;
+static_assert(kWppFarBytes % 16 == 0 && (size_t)kWppFarBytes * kWppLeftBps * kWppWarps <=
+                                            sizeof(int32_t) * kMpWarpsPerSm * kMpMembers * kMpCap,
+              "the near lists' part of the scratch");
 constexpr int kWppGrpLeaves = 448;   // leaf list of a group walk, shared by the group's particles
 constexpr int kWppGrpSpan = 64;      // default group span: one leaf-parent node (kLeaf * kFan particles)
 constexpr float kWppWalkR = 1.04f;   // default walk radius of the density pass (times the starting h)
