@@ -98,7 +98,7 @@ __device__ __forceinline__ float4 grav_join(int c0, int c1, uint4 c, float sf, Q
     return make_float4(sx * s, sy * s, sz * s, M);
 }
 
-// Moments of levels 0 to 2, a block per kTreeT leaves (as the bounds, see grid.cu).
+// Moments of levels 0 to 3, a block per kTreeT leaves (as the bounds, see grid.cu).
 __global__ void __launch_bounds__(kTreeT) k_grav_low(const uint4* __restrict__ posm, const BoxDesc* __restrict__ boxes,
                                                      const uint4* __restrict__ nc, float4* __restrict__ nm) {
     __shared__ float4 sq[kTreeT];

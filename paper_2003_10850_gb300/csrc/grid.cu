@@ -297,15 +297,140 @@ __global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* _
     }
 }
 
+// The whole sort in one block, for up to kRsSmall items: the passes follow one
+// another in shared memory, ranked and placed as k_rs_pass does. A set this small
+// is one or two tiles of the passes above, and pays their launches and round trips
+// through global memory (about 8 us each) for a microsecond or two of work:
+// 4,096 keys 70 -> 34 us.
+constexpr int kRsSmallT = 1024, kRsSmallWarps = kRsSmallT / 32;
+static_assert(kRsSmall == kRsSmallT * kRsIPT, "items of the block");
+struct RsSmallSmem {
+    unsigned long long key[kRsSmall];
+    unsigned val[kRsSmall];
+    unsigned short wcnt[kRsSmallWarps][kRsDig];
+    unsigned start[kRsDig];
+    unsigned wsum[kRsDig / 32];
+};
+__global__ void __launch_bounds__(kRsSmallT) k_rs_small(const unsigned long long* __restrict__ kin,
+                                                        unsigned long long* __restrict__ kout,
+                                                        unsigned* __restrict__ vout, int n, int passes) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    RsSmallSmem& sm = *reinterpret_cast<RsSmallSmem*>(raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int first = warp * (32 * kRsIPT) + lane;   // this lane's items: first + 32 r
+    const bool any = warp * (32 * kRsIPT) < n;       // the warp has items
+    unsigned long long key[kRsIPT];
+    unsigned val[kRsIPT], rank[kRsIPT];
+#pragma unroll
+    for (int r = 0; r < kRsIPT; ++r) {
+        val[r] = (unsigned)(first + 32 * r);
+        key[r] = first + 32 * r < n ? kin[first + 32 * r] : 0ull;
+    }
+    for (int pass = 0; pass < passes; ++pass) {
+        const int shift = pass * kRsBits;
+        {
+            unsigned* w = reinterpret_cast<unsigned*>(sm.wcnt[warp]);
+#pragma unroll
+            for (int k = 0; k < kRsDig / 64; ++k) w[k * 32 + lane] = 0u;
+        }
+        __syncwarp();
+        // places past n carry the last digit: behind every item in every pass
+        auto digit = [&](int r) {
+            return first + 32 * r < n ? (unsigned)(key[r] >> shift) & (kRsDig - 1u) : kRsDig - 1u;
+        };
+        if (any) {
+            unsigned peers[kRsIPT];
+#pragma unroll
+            for (int r = 0; r < kRsIPT; ++r) {
+                const unsigned d = digit(r);
+                unsigned m = 0xffffffffu;
+#pragma unroll
+                for (int b = 0; b < kRsBits; ++b) {
+                    const bool one = (d >> b) & 1u;
+                    const unsigned v = __ballot_sync(0xffffffffu, one);
+                    m &= one ? v : ~v;
+                }
+                peers[r] = m;
+            }
+#pragma unroll
+            for (int r = 0; r < kRsIPT; ++r) {
+                const unsigned d = digit(r), b = sm.wcnt[warp][d];
+                const unsigned before = __popc(peers[r] & ((1u << lane) - 1u));
+                __syncwarp();   // every lane has read its digit's count
+                if (before == 0u) sm.wcnt[warp][d] = (unsigned short)(b + __popc(peers[r]));
+                rank[r] = b + before;
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        unsigned cnt = 0u, x = 0u;
+        if (tid < kRsDig) {
+#pragma unroll
+            for (int w = 0; w < kRsSmallWarps; ++w) {
+                const unsigned c = sm.wcnt[w][tid];
+                sm.wcnt[w][tid] = (unsigned short)cnt;
+                cnt += c;
+            }
+            x = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) sm.wsum[warp] = x;
+        }
+        __syncthreads();
+        if (tid < kRsDig) {
+            unsigned before = 0u;
+#pragma unroll
+            for (int w = 0; w < kRsDig / 32; ++w) before += w < warp ? sm.wsum[w] : 0u;
+            sm.start[tid] = before + x - cnt;
+        }
+        __syncthreads();
+        if (any) {
+#pragma unroll
+            for (int r = 0; r < kRsIPT; ++r) {
+                const unsigned d = digit(r), q = sm.start[d] + sm.wcnt[warp][d] + rank[r];
+                sm.key[q] = key[r];
+                sm.val[q] = val[r];
+            }
+        }
+        __syncthreads();
+        if (any) {
+#pragma unroll
+            for (int r = 0; r < kRsIPT; ++r) {
+                key[r] = sm.key[first + 32 * r];
+                val[r] = sm.val[first + 32 * r];
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kRsIPT; ++r) {
+        if (first + 32 * r < n) {
+            kout[first + 32 * r] = key[r];
+            vout[first + 32 * r] = val[r];
+        }
+    }
+}
+
 // Sorts keys of key_bits bits with their indices. kin is read by the first
 // pass only (and not written); the passes write (ka, va), (kb, vb), (ka, va),
 // ... in turn, so an odd number of passes ends in (ka, va). With an odd number
-// kin may be kb, with an even number kin may not be ka.
+// kin may be kb, with an even number kin may not be ka. (Up to kRsSmall items go
+// straight to where the last pass would end.)
 cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsigned* va, unsigned long long* kb,
                     unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, Counters* ctr,
                     cudaStream_t s, unsigned* launches) {
     const int passes = (key_bits + kRsBits - 1) / kRsBits;
     const int tiles = (n + kRsTile - 1) / kRsTile;
+    if (n <= kRsSmall) {
+        cudaError_t e = cudaFuncSetAttribute(k_rs_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)sizeof(RsSmallSmem));
+        if (e) return e;
+        k_rs_small<<<1, kRsSmallT, sizeof(RsSmallSmem), s>>>(kin, passes & 1 ? ka : kb, passes & 1 ? va : vb, n, passes);
+        ++*launches;
+        return cudaGetLastError();
+    }
     unsigned* hist = reinterpret_cast<unsigned*>(work);
     unsigned* ticket = hist + kRsMaxPass * kRsDig;
     unsigned long long* status = reinterpret_cast<unsigned long long*>(work + kRsHead);
@@ -348,7 +473,7 @@ __device__ __forceinline__ void node_geom(uint4 a, uint4 b, double s, uint4& c, 
 }
 
 // The hierarchy is built in two launches: blocks of kTreeT leaves form levels
-// 0 to 2 of their part (a level's results pass through shared memory), then one
+// 0 to 3 of their part (a level's results pass through shared memory), then one
 // block per box forms the few nodes of the levels above, one level after another.
 // (One launch per level, most of them a handful of threads, took five to seven.)
 

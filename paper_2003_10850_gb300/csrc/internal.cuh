@@ -126,8 +126,8 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
                       sph_grid** out);
 void grid_free(sph_grid* g);
 // hierarchy passes: leaves per block of the first kernel, levels it forms, threads per box of the second
-constexpr int kTreeT = 256, kTreeLow = 3, kTreeTopT = 512;
-static_assert(kTreeT % (kFan * kFan) == 0, "whole level-2 nodes per block");
+constexpr int kTreeT = 512, kTreeLow = 4, kTreeTopT = 512;
+static_assert(kTreeT == kFan * kFan * kFan, "one level-3 node per block");
 // re-quantise, re-sort and rebuild the hierarchy in place (same n and boxes)
 sph_status grid_update(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s);
 // hmax of every node from the caller-order h
@@ -145,6 +145,7 @@ void flag_list(sph_grid* g, const uint8_t* flag, long long tick, int max_bin, in
 constexpr int kRsBits = 9;          // bits per pass
 constexpr int kRsTile = 4096;       // items per block
 constexpr int kRsMaxPass = 8;
+constexpr int kRsSmall = 8192;      // items that one block sorts by itself
 constexpr size_t kRsHead = sizeof(unsigned) * (kRsMaxPass * (1 << kRsBits) + 2 * kRsMaxPass);   // digit counts, tickets
 constexpr size_t rs_work_bytes(int64_t n) {
     return kRsHead + sizeof(unsigned long long) * (1 << kRsBits) * (size_t)((n + kRsTile - 1) / kRsTile);
