@@ -213,7 +213,8 @@ static sph_status density_call(sph_ctx* ctx, const sph_grid* grid, float* h, con
     cudaStream_t s = (cudaStream_t)stream;
     sph_grid* g = const_cast<sph_grid*>(grid);  // per-call scratch lives in the grid
     const Path path = pick_path(params->flags);
-    grid_active(g, active, n_active, s);
+    grid_active(g, active, n_active, s,
+                path == Path::Wpp ? density_begin(ctx, g, active != nullptr, na, params->flags) : CallBegin());
     DensityLaunch a;
     a.g = g;
     a.h = h;
@@ -285,7 +286,7 @@ static sph_status force_call(sph_ctx* ctx, const sph_grid* grid, const float* ve
     sph_grid* g = const_cast<sph_grid*>(grid);
     const Path path = pick_path(params->flags & ~SPH_DENSITY_BUFFERED);
     grid_refresh_hmax(g, h, s);
-    grid_active(g, active, n_active, s);
+    grid_active(g, active, n_active, s, path == Path::Wpp ? force_begin(ctx, g, na) : CallBegin());
     ForceLaunch a;
     a.g = g;
     a.vel = vel;
@@ -381,7 +382,10 @@ sph_status sph_gravity(sph_ctx* ctx, const sph_grid* grid, const int32_t* active
     if (cudaSetDevice(ctx->device)) return fail(ctx, SPH_ERR_CUDA, "cudaSetDevice failed");
     cudaStream_t s = (cudaStream_t)stream;
     sph_grid* g = const_cast<sph_grid*>(grid);
-    grid_active(g, active, n_active, s);
+    CallBegin b;
+    b.queue = ctx->queue;
+    b.queue_mask = 1u << 4;
+    grid_active(g, active, n_active, s, b);
     GravityLaunch L;
     L.g = g;
     L.G = gp->G;

@@ -583,8 +583,6 @@ cudaError_t launch_gravity(sph_ctx* ctx, const GravityLaunch& L, int64_t n_activ
     GravBox* gbox = reinterpret_cast<GravBox*>(g->grav_box);
     k_grav_box_rc<<<(nb + 127) / 128, 128, 0, s>>>(g->boxes, nb, L.r_cut, gbox);
     ++ctx->launches;
-    cudaError_t e = cudaMemsetAsync(ctx->queue + 4, 0, sizeof(unsigned), s);
-    if (e) return e;
     GravArgs a = {};
     a.boxes = g->boxes;
     a.n_boxes = nb;

@@ -505,19 +505,23 @@ __global__ void __launch_bounds__(kTreeT) k_tree_low(const uint4* __restrict__ p
     const uint4 a0 = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0), b0 = make_uint4(0, 0, 0, 0);
     uint4 a = a0, b = b0, c;
     if (t < B.lvl_n[0]) {
-        const long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
-        for (long long p = p0; p < p1; ++p) {
-            const uint4 x = posm[p];
-            join_bbox(a, b, x, x);
-        }
+        const long long p0 = B.off + (long long)t * kLeaf;
+        const int np = (int)min((long long)kLeaf, B.off + B.n - p0);
+        uint4 x[kLeaf];   // all loads in flight together
+#pragma unroll
+        for (int k = 0; k < kLeaf; ++k)
+            if (k < np) x[k] = posm[p0 + k];
+#pragma unroll
+        for (int k = 0; k < kLeaf; ++k)
+            if (k < np) join_bbox(a, b, x[k], x[k]);
         put_bbox(B.lvl_off[0] + t, a, b, s, lo, hi, nc, ne, c);
         // leaf-relative FP32 coordinates (box units) and mass of the leaf's particles
         const float sf = (float)s;
-        for (long long p = p0; p < p1; ++p) {
-            const uint4 x = posm[p];
-            posf[p] = make_float4((float)(int)(x.x - c.x) * sf, (float)(int)(x.y - c.y) * sf,
-                                  (float)(int)(x.z - c.z) * sf, __uint_as_float(x.w));
-        }
+#pragma unroll
+        for (int k = 0; k < kLeaf; ++k)
+            if (k < np)
+                posf[p0 + k] = make_float4((float)(int)(x[k].x - c.x) * sf, (float)(int)(x[k].y - c.y) * sf,
+                                           (float)(int)(x[k].z - c.z) * sf, __uint_as_float(x[k].w));
     }
     sa[tid] = a;
     sb[tid] = b;
@@ -565,8 +569,13 @@ __global__ void __launch_bounds__(kTreeT) k_hmax_low(const int32_t* __restrict__
     if (blockIdx.x * kTreeT >= B.lvl_n[0]) return;
     float m = 0.f;
     if (t < B.lvl_n[0]) {
-        const long long p0 = B.off + (long long)t * kLeaf, p1 = min(p0 + kLeaf, B.off + B.n);
-        for (long long p = p0; p < p1; ++p) m = fmaxf(m, h[perm[p]]);
+        const long long p0 = B.off + (long long)t * kLeaf;
+        const int np = (int)min((long long)kLeaf, B.off + B.n - p0);
+        float x[kLeaf];   // all gathers in flight together
+#pragma unroll
+        for (int k = 0; k < kLeaf; ++k) x[k] = k < np ? h[perm[p0 + k]] : 0.f;
+#pragma unroll
+        for (int k = 0; k < kLeaf; ++k) m = fmaxf(m, x[k]);
         hmax[B.lvl_off[0] + t] = m;
         ne[B.lvl_off[0] + t].w = m;
     }
@@ -610,11 +619,26 @@ __global__ void __launch_bounds__(kTreeTopT) k_hmax_top(const BoxDesc* __restric
 // a6: active list
 // ---------------------------------------------------------------------------
 
+// What a call clears before its kernels, in the launch that makes its active list
+// (each a memset or a launch of its own otherwise).
+__device__ __forceinline__ void call_begin(const CallBegin& b, int k) {
+    if (k < kQueues && ((b.queue_mask >> k) & 1u)) b.queue[k] = 0u;
+    if (b.list_zero && k < 2) b.list_zero[k] = 0u;
+    if (b.list_new) {   // a density call that records lists: clear the status words, one more generation
+        if (k < kListGen) b.list_new[k] = 0u;
+        else if (k == kListGen) b.list_new[kListGen] += 1u;
+    }
+}
+
 // all particles active: the identity list, and its length
-__global__ void k_iota_count(int32_t* a, int n, uint32_t* count) {
+__global__ void k_iota_count(int32_t* a, int n, uint32_t* count, CallBegin b) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) a[k] = k;
+    if (k < n) {
+        a[k] = k;
+        if (b.ext_n) b.ext_n[k] = 0u;
+    }
     if (k == 0) *count = (uint32_t)n;
+    if (blockIdx.x == 0) call_begin(b, k);
 }
 
 __global__ void k_mark(const int32_t* __restrict__ active, int na, const int32_t* __restrict__ rank,
@@ -637,9 +661,10 @@ constexpr int kCpT = 256, kCpPer = 16;
 static_assert(kCpTile == kCpT * kCpPer, "flags per block");
 __global__ void __launch_bounds__(kCpT) k_flag_list(const uint8_t* __restrict__ flag, int n, long long tick, int max_bin,
                                                     unsigned long long* work, int32_t* __restrict__ list,
-                                                    uint32_t* __restrict__ count, Counters* ctr) {
+                                                    uint32_t* __restrict__ count, Counters* ctr, CallBegin b) {
     __shared__ unsigned s_tile, s_before, s_warp[kCpT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.x == 0) call_begin(b, tid);
     if (tid == 0) s_tile = atomicAdd(reinterpret_cast<unsigned*>(work), 1u);
     __syncthreads();
     const int tile = (int)s_tile;
@@ -914,19 +939,19 @@ void grid_refresh_hmax(sph_grid* g, const float* h, cudaStream_t s) {
 }
 
 void flag_list(sph_grid* g, const uint8_t* flag, long long tick, int max_bin, int32_t* list, uint32_t* count,
-               cudaStream_t s) {
+               cudaStream_t s, const CallBegin& b) {
     const int n = (int)g->n;
     k_flag_list<<<(n + kCpTile - 1) / kCpTile, kCpT, 0, s>>>(flag, n, tick, max_bin,
                                                              (unsigned long long*)(g->flag + flag_bytes(n)), list, count,
-                                                             g->ctx->counters);
+                                                             g->ctx->counters, b);
     ++g->ctx->launches;
 }
 
-void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStream_t s) {
+void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStream_t s, const CallBegin& b) {
     int n = (int)g->n;
     unsigned& nl = g->ctx->launches;
     if (!active) {
-        k_iota_count<<<(n + 255) / 256, 256, 0, s>>>(g->act, n, g->act_n);
+        k_iota_count<<<(n + 255) / 256, 256, 0, s>>>(g->act, n, g->act_n, b);
         ++nl;
     } else {
         cudaMemsetAsync(g->flag, 0, flag_bytes(n) + flag_work_bytes(n), s);   // flags and flag_list's words
@@ -935,7 +960,8 @@ void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStrea
                                                                   g->ctx->counters);
             ++nl;
         }
-        flag_list(g, g->flag, 0, -1, g->act, g->act_n, s);
+        if (b.ext_n) cudaMemsetAsync(b.ext_n, 0, sizeof(uint32_t) * n, s);
+        flag_list(g, g->flag, 0, -1, g->act, g->act_n, s, b);
     }
 }
 

@@ -132,15 +132,26 @@ static_assert(kTreeT == kFan * kFan * kFan, "one level-3 node per block");
 sph_status grid_update(sph_grid* g, const void* pos, int f64, const float* mass, cudaStream_t s);
 // hmax of every node from the caller-order h
 void grid_refresh_hmax(sph_grid* g, const float* h, cudaStream_t s);
-// active list: sorted indices in g->act, count in *g->act_n
-void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStream_t s);
 // The set flags' indices, ascending, in list and their number in *count. The words
 // behind g->flag must be clear; flag as k_flag_list in grid.cu.
 constexpr int kCpTile = 4096;
 constexpr size_t flag_bytes(int64_t n) { return ((size_t)n + 15) / 16 * 16; }
 constexpr size_t flag_work_bytes(int64_t n) { return 8 * ((size_t)(n + kCpTile - 1) / kCpTile + 1); }
+// What a call clears before its kernels, in the launch that makes its active list: its
+// words of the context's queue, two status words of the lists (force), the lists'
+// status words and counts with a new generation (a density call that records).
+struct CallBegin {
+    unsigned* queue = nullptr;
+    unsigned queue_mask = 0u;
+    unsigned* list_zero = nullptr;
+    unsigned* list_new = nullptr;
+    uint32_t* ext_n = nullptr;   // n
+};
 void flag_list(sph_grid* g, const uint8_t* flag, long long tick, int max_bin, int32_t* list, uint32_t* count,
-               cudaStream_t s);
+               cudaStream_t s, const CallBegin& b = CallBegin());
+// active list: sorted indices in g->act, count in *g->act_n
+void grid_active(sph_grid* g, const int32_t* active, int64_t n_active, cudaStream_t s,
+                 const CallBegin& b = CallBegin());
 // stable radix sort of (key, index) pairs, see grid.cu; work: rs_work_bytes(n) bytes, 16-byte aligned
 constexpr int kRsBits = 9;          // bits per pass
 constexpr int kRsTile = 4096;       // items per block
@@ -241,6 +252,9 @@ cudaError_t launch_gravity(sph_ctx* ctx, const GravityLaunch& L, int64_t n_activ
 
 // wpp_density.cu, wpp_force.cu (one warp per particle)
 cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_active, cudaStream_t s);
+// what such a call clears first
+CallBegin density_begin(sph_ctx* ctx, const sph_grid* g, bool active_list, int64_t n_active, int flags);
+CallBegin force_begin(sph_ctx* ctx, const sph_grid* g, int64_t n_active);
 cudaError_t launch_force_wpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_active, cudaStream_t s);
 
 // f64.cu (SPH_FP64)

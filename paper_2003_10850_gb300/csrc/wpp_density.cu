@@ -1255,14 +1255,6 @@ __global__ void __launch_bounds__(256) k_list_sort(int n, int per, int32_t* __re
     }
 }
 
-// Start of a density call that records lists: clear the status words, one
-// more generation (the stamp of the lists this call writes).
-__global__ void k_list_begin(unsigned* list_st) {
-    const int t = (int)threadIdx.x;
-    if (t < kListGen) list_st[t] = 0u;
-    else if (t == kListGen) list_st[kListGen] += 1u;
-}
-
 // A call on part of the particles: the h every inactive particle keeps (with
 // its position, in sorted order) for the extra-partner tests, and the h of
 // the inactive particles alone in caller order (0 for the active ones) for the
@@ -1288,10 +1280,49 @@ __global__ void k_vel_pack(int n, const int32_t* __restrict__ perm, const float*
     vm[p] = make_float4(vel[3 * o], vel[3 * o + 1], vel[3 * o + 2], posf[p].w);
 }
 
+// How a call runs: the member-parallel kernel first or the one-particle kernel
+// alone, and which lists it records.
+//
+// Neighbour lists for the force pass, each stamped with this call's
+// generation. A call whose active set can cover every particle (no list,
+// or a list of n entries) records them whatever the kernel; they serve a
+// force call only if every particle was in fact active (checked on the
+// device: the list count and the lists written both equal n). With
+// SPH_PARTIAL_LISTS, a call on an active list (padded or not) that runs the
+// member-parallel kernel records the active particles' lists and also
+// finds their extra partners among the inactive ones.
+// (The partial lists need the member-parallel kernel: with the flag it runs
+// for any active set that is not too sparse to form groups.)
+struct DensityPlan {
+    bool scratch, mp, part, rec;
+};
+static DensityPlan density_plan(const sph_ctx* ctx, const sph_grid* g, bool active_list, int64_t n_active, bool flag) {
+    DensityPlan p;
+    // the scratch holds kMpWarpsPerSm warps per SM of the device the grid was built on
+    p.scratch = g->ctx->sm_count >= ctx->sm_count && g->mp_j != nullptr;
+    const bool want_part = g->nbr != nullptr && active_list && flag && n_active * 256 >= g->n;
+    p.mp = (want_part || wpp_groups_pay(ctx, n_active, g->n)) && p.scratch;
+    p.part = want_part && p.mp;
+    p.rec = p.part || (g->nbr != nullptr && n_active == g->n);
+    return p;
+}
+
+CallBegin density_begin(sph_ctx* ctx, const sph_grid* g, bool active_list, int64_t n_active, int flags) {
+    const DensityPlan p = density_plan(ctx, g, active_list, n_active, (flags & SPH_PARTIAL_LISTS) != 0);
+    CallBegin b;
+    b.queue = ctx->queue;
+    b.queue_mask = 1u << 2;
+    if (p.mp) b.queue_mask |= 1u << 5 | 1u << 6;
+    if (p.rec) {
+        b.list_new = g->list_st;
+        b.ext_n = g->ext_n;
+    }
+    return b;
+}
+
 cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_active, cudaStream_t s) {
     sph_grid* g = const_cast<sph_grid*>(a.g);
-    cudaError_t e = cudaMemsetAsync(ctx->queue + 2, 0, sizeof(unsigned), s);
-    if (e) return e;
+    cudaError_t e;
     WppArgs c = wpp_common(ctx, g, ctx->queue + 2);
     int blocks = 0;
     const int bps = std::min(a.blocks_per_sm > 0 ? a.blocks_per_sm : kWppDensityBps, kWppDensityMaxBps);
@@ -1309,8 +1340,8 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
     c.fixed_h = a.fixed_h;
     c.walk_r = a.walk_radius > 0.0 ? (float)a.walk_radius : kWppWalkR;
     c.grp_shift = wpp_grp_shift(a.group_span);
-    // the scratch holds kMpWarpsPerSm warps per SM of the device the grid was built on
-    c.mp_j = g->ctx->sm_count >= ctx->sm_count ? g->mp_j : nullptr;
+    const DensityPlan plan = density_plan(ctx, g, a.active_list, n_active, a.partial_lists);
+    c.mp_j = plan.scratch ? g->mp_j : nullptr;
     if (a.divv) {
         k_vel_pack<<<(int)((g->n + 255) / 256), 256, 0, s>>>((int)g->n, g->perm, a.vel, g->posf, g->fvm);
         ++ctx->launches;
@@ -1318,20 +1349,7 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
         c.divv = a.divv;
         c.curlv = a.curlv;
     }
-    // Neighbour lists for the force pass, each stamped with this call's
-    // generation. A call whose active set can cover every particle (no list,
-    // or a list of n entries) records them whatever the kernel; they serve a
-    // force call only if every particle was in fact active (checked on the
-    // device: the list count and the lists written both equal n). With
-    // SPH_PARTIAL_LISTS, a call on an active list (padded or not) that runs the
-    // member-parallel kernel records the active particles' lists and also
-    // finds their extra partners among the inactive ones.
-    // (The partial lists need the member-parallel kernel: with the flag it runs
-    // for any active set that is not too sparse to form groups.)
-    const bool want_part = g->nbr != nullptr && a.active_list && a.partial_lists && n_active * 256 >= g->n;
-    const bool mp_path = (want_part || wpp_groups_pay(ctx, n_active, g->n)) && c.mp_j != nullptr;
-    const bool part = want_part && mp_path;
-    const bool rec = part || (g->nbr != nullptr && n_active == g->n);
+    const bool mp_path = plan.mp, part = plan.part, rec = plan.rec;
     if (rec) {
         c.nbr = g->nbr;
         c.nbr_off = g->nbr_off;
@@ -1345,9 +1363,6 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
         // chunks small enough that every warp's first reservations fit in a quarter of the pool
         const long long warps = (long long)blocks * kWppWarps;
         c.list_chunk = (int)std::max<long long>(32, std::min<long long>(kListChunk, g->list_pool / (4 * warps)));
-        k_list_begin<<<1, 32, 0, s>>>(g->list_st);
-        ++ctx->launches;
-        if ((e = cudaMemsetAsync(g->ext_n, 0, sizeof(uint32_t) * g->n, s))) return e;
         if (part) {
             const int n = (int)g->n;
             k_list_snap<<<(n + 255) / 256, 256, 0, s>>>(n, g->perm, a.h, g->posm, g->flag, g->list_xh, g->st_lo);
@@ -1371,7 +1386,6 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
     } else {
         // leftovers of the member-parallel kernel: list g->den_left, count queue[6],
         // work queue queue[5]
-        if ((e = cudaMemsetAsync(ctx->queue + 5, 0, 2 * sizeof(unsigned), s))) return e;
         c.left = g->den_left;
         c.left_n = ctx->queue + 6;
         // whole groups per queue grab, whatever the active count: a warp's

@@ -693,15 +693,27 @@ static void launch_force_walk(bool hash, bool six, int visc, bool cond, int bloc
     else hash ? launch_fw<true, 8>(visc, cond, blocks, s, c) : launch_fw<false, 8>(visc, cond, blocks, s, c);
 }
 
+static bool force_groups(const sph_ctx* ctx, const sph_grid* g, int64_t n_active) {
+    // (the pair-list scratch is sized for the context the grid was built with)
+    return g->ctx->sm_count >= ctx->sm_count && wpp_groups_pay(ctx, n_active, g->n, kFmMinWarps);
+}
+
+CallBegin force_begin(sph_ctx* ctx, const sph_grid* g, int64_t n_active) {
+    CallBegin b;
+    b.queue = ctx->queue;
+    b.queue_mask = 1u << 3;
+    if (force_groups(ctx, g, n_active)) b.queue_mask |= 1u << 6 | 1u << 7;
+    if (g->nbr && g->lists_rec) b.list_zero = g->list_st + 2;
+    return b;
+}
+
 cudaError_t launch_force_wpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_active, cudaStream_t s) {
     sph_grid* g = const_cast<sph_grid*>(a.g);
     cudaError_t e;
     const bool lists = g->nbr != nullptr && g->lists_rec;
-    if (lists && (e = cudaMemsetAsync(g->list_st + 2, 0, 2 * sizeof(unsigned), s))) return e;
     force_pack(g, a.vel, a.u, a.h, a.rho, a.omega, (float)a.gamma, s, lists ? g->list_xh : nullptr,
                lists ? g->list_st + 2 : nullptr, a.divv, a.curlv, a.kappa, a.alpha_v);
     ++ctx->launches;
-    if ((e = cudaMemsetAsync(ctx->queue + 3, 0, sizeof(unsigned), s))) return e;
     WppArgs c = wpp_common(ctx, g, ctx->queue + 3);
     c.grp_shift = wpp_grp_shift(a.group_span);
     int blocks = 0;
@@ -745,8 +757,7 @@ cudaError_t launch_force_wpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_activ
     // the walk: member-parallel for groups (nothing to do when the lists served
     // the call), then one particle per warp for what it leaves and for the
     // particles the lists could not serve
-    if (g->ctx->sm_count >= ctx->sm_count && wpp_groups_pay(ctx, n_active, g->n, kFmMinWarps)) {
-        if ((e = cudaMemsetAsync(ctx->queue + 6, 0, 2 * sizeof(unsigned), s))) return e;
+    if (force_groups(ctx, g, n_active)) {
         WppArgs cm = c;
         c.mp_min = cm.mp_min = wpp_mp_min(ctx, kFmMinWarps);
         cm.mp_j = g->mp_j;
