@@ -462,11 +462,9 @@ __global__ void __launch_bounds__(kBwThreads) k_backward(BwArgs a) {
 cudaError_t run_backward(sph_ctx* ctx, sph_grid* g, const BackwardLaunch& b, cudaStream_t s) {
     const int n = (int)g->n;
     if (!g->bw_ga) {
-        cudaError_t e = cudaSuccess;
-        if (!e) e = cudaMalloc(&g->bw_ga, sizeof(float4) * n);
-        if (!e) e = cudaMalloc(&g->bw_xbar, sizeof(float4) * n);
-        if (!e) e = cudaMalloc(&g->bw_rd, sizeof(float4) * n);
-        if (!e) e = cudaMalloc(&g->bw_f, sizeof(float) * 6 * (size_t)n);
+        const Part parts[] = {{&g->bw_ga, sizeof(float4) * n}, {&g->bw_xbar, sizeof(float4) * n},
+                              {&g->bw_rd, sizeof(float4) * n}, {&g->bw_f, sizeof(float) * 6 * (size_t)n}};
+        const cudaError_t e = carve(&g->bw_arena, parts);
         if (e) return e;
     }
     grid_refresh_hmax(g, b.h, s);

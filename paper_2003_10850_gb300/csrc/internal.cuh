@@ -91,6 +91,10 @@ struct sph_grid {
     int32_t* mp_x = nullptr;               // density, member-parallel path of a partial call: per warp,
                                            // kMpMembers x kMpFar inactive partners beyond the near radius
     int64_t list_pool = 0;                 // entries of the nbr pool
+    // the allocations that hold the arrays above and below
+    void* arena = nullptr;
+    void* list_arena = nullptr;
+    void* bw_arena = nullptr;
     // adjoint scratch (allocated by the first sph_backward on the grid)
     float4* bw_ga = nullptr;
     float4* bw_xbar = nullptr;
@@ -125,6 +129,16 @@ sph_status grid_build(sph_ctx* ctx, const void* pos, int f64, const float* mass,
                       const int64_t* offs, const double* Ls, int nb, cudaStream_t s,
                       sph_grid** out);
 void grid_free(sph_grid* g);
+// one allocation for several arrays, each on a 256-byte boundary
+struct Part {
+    void** ptr;
+    size_t bytes;
+    template <typename T>
+    Part(T** p, size_t b) : ptr(reinterpret_cast<void**>(p)), bytes(b) {}
+};
+cudaError_t carve(void** base, const Part* parts, int n);
+template <int N>
+cudaError_t carve(void** base, const Part (&parts)[N]) { return carve(base, parts, N); }
 // hierarchy passes: leaves per block of the first kernel, levels it forms, threads per box of the second
 constexpr int kTreeT = 512, kTreeLow = 4, kTreeTopT = 512;
 static_assert(kTreeT == kFan * kFan * kFan, "one level-3 node per block");
