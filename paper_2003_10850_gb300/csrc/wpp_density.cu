@@ -587,7 +587,9 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
     }
 }
 
-template <bool HASH, int MINB, bool DIVCURL>
+// GROUP false: particles come one at a time (a.chunk 1), and the code of the shared
+// walks is left out: the kernel is large enough to miss the instruction cache.
+template <bool HASH, int MINB, bool DIVCURL, bool GROUP>
 __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
     __shared__ WppSmem smem[kWppWarps];
     WppSmem& sm = smem[threadIdx.x >> 5];
@@ -630,7 +632,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
                     hl = wpp_guess_h(B, a.node_lo, a.node_hi, G.p, ldexp(B.L, -32), a.n_target);
             }
             int ngl = -1;
-            if (G.n >= 2 && B.nlev > 1) {
+            if (GROUP && G.n >= 2 && B.nlev > 1) {
                 const float Rg = warp_max(a.fixed_h ? hl : hl * a.walk_r);
                 ngl = wpp_group_leaves(sm, B, a.node_c, a.node_e, Xl, G.p >= 0, sf, [&](float4) { return Rg; });
             }
@@ -768,7 +770,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
                         nnear = 0;
                         complete = true;
                         // a walk that overflows the leaf list evaluates its leaves at h as it goes
-                        if (first && ngl >= 0)
+                        if (GROUP && first && ngl >= 0)
                             wpp_filter(sm, ngl, B, a.node_c, a.node_e, Xi, sf, nlf, complete,
                                        [&](float4) { return Rw; }, [&]() { process(false); nlf = 0; });
                         else
@@ -1375,12 +1377,17 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
     WppSpan sp;
     if ((e = span_begin(ctx, a.time_kernels, 0, s, sp))) return e;
     const bool dc = a.divv != nullptr;
+    auto one = [&](auto group) {
+        constexpr bool G = decltype(group)::value;
+        constexpr int M = kWppLeftBps;
+        return a.hash ? (dc ? k_density_wpp<true, M, true, G> : k_density_wpp<true, M, false, G>)
+                      : (dc ? k_density_wpp<false, M, true, G> : k_density_wpp<false, M, false, G>);
+    };
     if (!mp_path) {
         // sparse active sets form groups of one: the one-particle kernel alone
-        auto k1 = a.hash ? (dc ? k_density_wpp<true, kWppLeftBps, true> : k_density_wpp<true, kWppLeftBps, false>)
-                         : (dc ? k_density_wpp<false, kWppLeftBps, true> : k_density_wpp<false, kWppLeftBps, false>);
         int b1 = 0;
         wpp_shape(ctx, kWppLeftBps, n_active, b1, c.chunk);
+        auto k1 = c.chunk > 1 ? one(std::true_type()) : one(std::false_type());
         k1<<<b1, kWppThreads, 0, s>>>(c);
         ++ctx->launches;
     } else {
@@ -1416,8 +1423,7 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
         cl.list_chunk = 0;
         int lblocks = 0, lchunk = 0;
         wpp_shape(ctx, kWppLeftBps, n_active, lblocks, lchunk);
-        auto kl = a.hash ? (dc ? k_density_wpp<true, kWppLeftBps, true> : k_density_wpp<true, kWppLeftBps, false>)
-                         : (dc ? k_density_wpp<false, kWppLeftBps, true> : k_density_wpp<false, kWppLeftBps, false>);
+        auto kl = one(std::false_type());
         kl<<<lblocks, kWppThreads, 0, s>>>(cl);
         ctx->launches += 2;
     }
