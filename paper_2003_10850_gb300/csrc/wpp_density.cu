@@ -198,57 +198,36 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                     const float mj = __uint_as_float(__float_as_uint(f0.w) & 0x7fffffffu);
                     const bool ina = PART && cand && Tj >= 0.f;
                     const bool anyina = PART && __any_sync(0xffffffffu, ina);
-                    if (!__any_sync(0xffffffffu, wide)) {
+                    // a wide leaf among them: exact integer separations from each member there
+                    const bool anyw = __any_sync(0xffffffffu, wide);
+                    const uint4 Xq = wide ? a.posm[q] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-                        for (int m = 0; m < kMpMembers; ++m) {
-                            const float4 g = mp.mem[m];
-                            const float dx = f0.x - g.x, dy = f0.y - g.y, dz = f0.z - g.z;
-                            const float r2 = dx * dx + dy * dy + dz * dz;
-                            const bool in = cand && q != mp.pm[m] && r2 < g.w;
-                            const unsigned msk = __ballot_sync(0xffffffffu, in);
-                            const int k = (cntm[m] & 0xffff) + __popc(msk & lt);
-                            if (in && k < kMpCap) {
-                                mp.d[m][k] = make_float2(r2, mj);
-                                mpj[m * kMpCap + k] = q;
-                            }
-                            cntm[m] += __popc(msk);
-                            if (anyina) {
-                                const bool far = ina && m < G.n && !(r2 < g.w) && r2 < Tj;
-                                const unsigned fm = __ballot_sync(0xffffffffu, far);
-                                const int kf = (cntm[m] >> 16) + __popc(fm & lt);
-                                if (far && kf < kMpFar) mpx[m * kMpFar + kf] = q;
-                                cntm[m] += __popc(fm) << 16;
-                            }
-                        }
-                    } else {
-                        // a wide leaf among them: exact integer separations from each member there
-                        const uint4 Xq = wide ? a.posm[q] : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                        for (int m = 0; m < kMpMembers; ++m) {
-                            const float4 g = mp.mem[m];
-                            float dx = f0.x - g.x, dy = f0.y - g.y, dz = f0.z - g.z;
+                    for (int m = 0; m < kMpMembers; ++m) {
+                        const float4 g = mp.mem[m];
+                        float dx = f0.x - g.x, dy = f0.y - g.y, dz = f0.z - g.z;
+                        if (anyw) {
                             if (wide) {
                                 const uint4 Xm = mp.X[m];
                                 dx = (float)(int)(Xq.x - Xm.x) * sf;
                                 dy = (float)(int)(Xq.y - Xm.y) * sf;
                                 dz = (float)(int)(Xq.z - Xm.z) * sf;
                             }
-                            const float r2 = dx * dx + dy * dy + dz * dz;
-                            const bool in = cand && q != mp.pm[m] && r2 < g.w;
-                            const unsigned msk = __ballot_sync(0xffffffffu, in);
-                            const int k = (cntm[m] & 0xffff) + __popc(msk & lt);
-                            if (in && k < kMpCap) {
-                                mp.d[m][k] = make_float2(r2, mj);
-                                mpj[m * kMpCap + k] = q;
-                            }
-                            cntm[m] += __popc(msk);
-                            if (anyina) {
-                                const bool far = ina && m < G.n && !(r2 < g.w) && r2 < Tj;
-                                const unsigned fm = __ballot_sync(0xffffffffu, far);
-                                const int kf = (cntm[m] >> 16) + __popc(fm & lt);
-                                if (far && kf < kMpFar) mpx[m * kMpFar + kf] = q;
-                                cntm[m] += __popc(fm) << 16;
-                            }
+                        }
+                        const float r2 = dx * dx + dy * dy + dz * dz;
+                        const bool in = cand && q != mp.pm[m] && r2 < g.w;
+                        const unsigned msk = __ballot_sync(0xffffffffu, in);
+                        const int k = (cntm[m] & 0xffff) + __popc(msk & lt);
+                        if (in && k < kMpCap) {
+                            mp.d[m][k] = make_float2(r2, mj);
+                            mpj[m * kMpCap + k] = q;
+                        }
+                        cntm[m] += __popc(msk);
+                        if (anyina) {
+                            const bool far = ina && m < G.n && !(r2 < g.w) && r2 < Tj;
+                            const unsigned fm = __ballot_sync(0xffffffffu, far);
+                            const int kf = (cntm[m] >> 16) + __popc(fm & lt);
+                            if (far && kf < kMpFar) mpx[m * kMpFar + kf] = q;
+                            cntm[m] += __popc(fm) << 16;
                         }
                     }
                 };
@@ -258,9 +237,11 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                 uint4 C_n;
                 float4 f_n;
                 fetch(0, e_n, q_n, cand_n, C_n, f_n);
-                for (int base = 0; base < ngl; base += 4) {
+                // (one place calls members(), the last candidates included: its code is long)
+                for (int base = 0;; base += 4) {
+                    const bool more = base < ngl;
                     const int e = e_n, q = q_n;
-                    const bool cand = cand_n;
+                    const bool cand = more && cand_n;
                     const uint4 C = C_n;
                     const float4 f = f_n;
                     if (base + 4 < ngl) fetch(base + 4, e_n, q_n, cand_n, C_n, f_n);
@@ -293,8 +274,8 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                         if (PART) mp.bt[slot] = Tj;
                     }
                     nb += __popc(pb);
-                    if (nb >= 32) {
-                        members(32);
+                    if (nb >= 32 || (!more && nb > 0)) {
+                        members(min(nb, 32));
                         if (pass && slot >= 32) {
                             mp.bp[slot - 32] = ent;
                             mp.bq[slot - 32] = q;
@@ -302,8 +283,8 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                         }
                         nb -= 32;
                     }
+                    if (!more) break;
                 }
-                if (nb > 0) members(nb);
                 if (lane == 0) c_tests += (unsigned long long)ctest * (unsigned)G.n;
                 __syncwarp();
                 // ---------------- h iteration: lanes 4m..4m+3 serve member m ----------------

@@ -509,9 +509,11 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
                 uint4 C_n;
                 float4 f_n;
                 fetch(0, e_n, q_n, cand_n, C_n, f_n);
-                for (int base = 0; base < ngl; base += 4) {
+                // (one place calls members(), the last candidates included: its code is long)
+                for (int base = 0;; base += 4) {
+                    const bool more = base < ngl;
                     const int e = e_n, q = q_n;
-                    const bool cand = cand_n;
+                    const bool cand = more && cand_n;
                     const uint4 C = C_n;
                     const float4 f = f_n;
                     if (base + 4 < ngl) fetch(base + 4, e_n, q_n, cand_n, C_n, f_n);
@@ -537,16 +539,16 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
                         sm.bq[slot] = q;
                     }
                     nb += __popc(pb);
-                    if (nb >= 32) {
-                        members(32);
+                    if (nb >= 32 || (!more && nb > 0)) {
+                        members(min(nb, 32));
                         if (pass && slot >= 32) {
                             sm.bp[slot - 32] = ent;
                             sm.bq[slot - 32] = q;
                         }
                         nb -= 32;
                     }
+                    if (!more) break;
                 }
-                if (nb > 0) members(nb);
                 if (lane == 0) c_tests += (unsigned long long)ctest * (unsigned)G.n;
                 // members whose list overflowed go to the one-particle walk
                 todo = 0;
