@@ -164,8 +164,8 @@ struct WppArgs {
     // density, member-parallel path: near-list indices, kMpMembers x kMpCap per persistent warp
     int32_t* mp_j;
     // density: the particles the member-parallel kernel leaves to the one-particle kernel
-    int32_t* left;
-    unsigned* left_n;
+    int32_t* left;               // density: the slow ones from the front (left_n[0] of them), the others
+    unsigned* left_n;            // from the back (left_n[1])
     // force: the member-parallel kernel's rule on the device's own active count
     // (wpp_groups_pay; 0: none); when it fails the one-particle kernel takes the whole set
     int mp_min;

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                                        [&](float4 e) { return PART ? fmaxf(Rg, e.w) : Rg; }, gg);
             }
             unsigned todo = (1u << G.n) - 1u;   // members left for the one-particle path
+            unsigned slow = todo;               // of these, the ones beside a compact clump (a list overflowed)
             if (ngl >= 0 && mpj && G.n >= 2) {
                 // ---------------- candidates: one sweep of the group's leaves ----------------
                 // 32 candidates per step (the next step's loaded while this one's are
@@ -533,6 +534,10 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                 todo = 0;
 #pragma unroll
                 for (int k = 0; k < kMpMembers; ++k) todo |= ((rb >> (4 * k)) & 1u) << k;
+                const unsigned sb = __ballot_sync(0xffffffffu, mval && cm > kMpCap && sub == 0);
+                slow = 0;
+#pragma unroll
+                for (int k = 0; k < kMpMembers; ++k) slow |= ((sb >> (4 * k)) & 1u) << k;
                 const float hnow = __shfl_sync(0xffffffffu, h, (int)(lane & 7u) * 4);
                 if ((int)lane < G.n && ((todo >> lane) & 1u)) hl = hnow;
                 __syncwarp();
@@ -540,12 +545,16 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
             // the members left over go to the one-particle kernel, each with the h
             // it should start from
             if (todo) {
-                const int nl = __popc(todo);
+                // the slow ones are taken first: one started last would run alone
+                const unsigned fast = todo & ~slow;
+                slow &= todo;
                 unsigned o = 0;
-                if (lane == 0) o = atomicAdd(a.left_n, (unsigned)nl);
-                o = __shfl_sync(0xffffffffu, o, 0);
+                if (lane == 0 && slow) o = atomicAdd(a.left_n, (unsigned)__popc(slow));
+                if (lane == 1 && fast) o = atomicAdd(a.left_n + 1, (unsigned)__popc(fast));
+                const unsigned os = __shfl_sync(0xffffffffu, o, 0), of = __shfl_sync(0xffffffffu, o, 1);
                 if ((int)lane < G.n && ((todo >> lane) & 1u)) {
-                    a.left[o + __popc(todo & lt)] = G.p;
+                    const bool sl = (slow >> lane) & 1u;
+                    a.left[sl ? (int)(os + __popc(slow & lt)) : a.n_total - 1 - (int)(of + __popc(fast & lt))] = G.p;
                     a.h[ol] = hl;
                     // PART: the one-particle kernel finds no far partners; the force pass walks for it
                     if (PART) a.ext_n[G.p] = (unsigned)kExtCap + 1u;
@@ -578,7 +587,9 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
     const unsigned lt = (1u << lane) - 1u;
     const float rel = 9.5367431640625e-07f;  // 2^-20
     const float nt = (float)a.n_target, nt3 = 3.f * nt, tol3 = 3.f * (float)a.n_tol;
-    const int cnt = (int)*a.count_ptr;
+    // leftovers (a.left): the slow ones at the front of the list, then the others from its end
+    const int nslow = a.left ? (int)a.left_n[0] : 0;
+    const int cnt = a.left ? nslow + (int)a.left_n[1] : (int)*a.count_ptr;
     if (cnt == 0) return;   // (before thousands of warps queue for nothing)
     unsigned c_pairs = 0, c_evals = 0, c_tests = 0, c_status = 0, c_lists = 0;   // per warp (32-bit suffices)
     long long ch_next = 0, ch_end = 0;   // the warp's current chunk of the neighbour-list pool
@@ -595,7 +606,9 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_wpp(WppArgs a) {
         if (t0 >= cnt) break;
         const int t1 = min(t0 + a.chunk, cnt);
         for (int t = t0; t < t1;) {
-            const WppGroup G = wpp_group(a.boxes, a.n_boxes, a.act, t, t1, a.grp_shift);
+            // (leftovers come one at a time, act[t] the only entry read)
+            const int32_t* act = a.left && t >= nslow ? a.left + (a.n_total - 1 - (t - nslow)) - t : a.act;
+            const WppGroup G = wpp_group(a.boxes, a.n_boxes, act, t, t1, a.grp_shift);
             t += G.n;
             const BoxDesc& B = a.boxes[G.box];
             const float sf = B.sf;
@@ -1295,7 +1308,7 @@ CallBegin density_begin(sph_ctx* ctx, const sph_grid* g, bool active_list, int64
     CallBegin b;
     b.queue = ctx->queue;
     b.queue_mask = 1u << 2;
-    if (p.mp) b.queue_mask |= 1u << 5 | 1u << 6;
+    if (p.mp) b.queue_mask |= 1u << 5 | 1u << 6 | 1u << 7;
     if (p.rec) {
         b.list_new = g->list_st;
         b.ext_n = g->ext_n;
@@ -1372,8 +1385,8 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
         k1<<<b1, kWppThreads, 0, s>>>(c);
         ++ctx->launches;
     } else {
-        // leftovers of the member-parallel kernel: list g->den_left, count queue[6],
-        // work queue queue[5]
+        // leftovers of the member-parallel kernel: list g->den_left, counts queue[6] and
+        // queue[7], work queue queue[5]
         c.left = g->den_left;
         c.left_n = ctx->queue + 6;
         // whole groups per queue grab, whatever the active count: a warp's
@@ -1395,7 +1408,6 @@ cudaError_t launch_density_wpp(sph_ctx* ctx, const DensityLaunch& a, int64_t n_a
         // member-parallel kernel left for them
         WppArgs cl = c;
         cl.act = g->den_left;
-        cl.count_ptr = ctx->queue + 6;
         cl.queue = ctx->queue + 5;
         cl.chunk = 1;
         cl.guess_h = 0;
