@@ -22,9 +22,12 @@
 //
 // A warp walks for a group of up to M active particles (its members) of one
 // aligned run of 64 sorted particles, 32/M lanes serving each member:
-// - a step pops up to four opened nodes and tests their children, one per lane,
-//   against every member, in FP32 where that settles the exact rule and by the
-//   rule itself elsewhere (see grav_decide); a child that some member opens is
+// - a step pops up to four opened nodes, one child per lane; with four or more
+//   members the children beyond every member's cutoff go (by the members' box, in
+//   FP32 with a margin) and the others wait until there are 32;
+// - 32 children, one per lane, are tested against every member, in FP32 where that
+//   settles the exact rule and by the rule itself elsewhere (see grav_decide); a
+//   child that some member opens is
 //   pushed with its member mask, and a member that accepts a node or opens a leaf
 //   puts it on its own list;
 // - a full list is worked off by the lanes of its member: accepted nodes, and the
@@ -44,10 +47,10 @@ constexpr int kGravStack = 256;   // see the bound below
 constexpr int kGravLeaves = 128;  // opened leaves waiting per member; a step adds <= 32
 constexpr int kGravNodes = 64;    // accepted nodes waiting per member; a step adds <= 32
 
-// Stack bound: a pop-4 step starts at sp <= 96 and pushes <= 32 children; in
-// the pop-1 regime a step pushes <= 8 children of the node it pops, so the
-// stack grows by at most 7 per level of depth-first descent:
-// sp <= 124 + 7 kMaxLev < kGravStack.
+// Stack bound: the 32 children tested after pop-4 steps from sp <= 96 push <= 32, and
+// the <= 31 still waiting then go before the next pop: sp <= 155. In the pop-1
+// regime the children of a node are tested at once (<= 8 pushed), so the stack grows
+// by at most 7 per level of depth-first descent: sp <= 155 + 7 kMaxLev < kGravStack.
 
 struct GravBox {
     unsigned long long RCi;
@@ -342,6 +345,8 @@ struct GravSmem {
     uint4 mX[M];                     // member integer positions
     int lf[M][kGravLeaves];          // opened leaves (first particle)
     int nd[M][kGravNodes];           // accepted nodes (global index)
+    int qe[M >= 4 ? 64 : 1];         // children waiting for the members' tests (level, index)
+    unsigned char qm[M >= 4 ? 64 : 1];
 };
 
 template <int M>
@@ -416,6 +421,27 @@ __global__ void __launch_bounds__(kWppThreads, 5) k_gravity(GravArgs a) {
                 kahan_add(Sz, Cz, az.x + az.y);
                 ax = ay = az = both(0.f);
             };
+            // the members' box: centre, half extents (integer units, rounded up)
+            uint4 Gc = make_uint4(0u, 0u, 0u, 0u);
+            float gex = 0.f, gey = 0.f, gez = 0.f;
+            bool gok = false;
+            if (M >= 4) {
+                const unsigned X0x = __shfl_sync(0xffffffffu, Xl.x, 0), X0y = __shfl_sync(0xffffffffu, Xl.y, 0),
+                               X0z = __shfl_sync(0xffffffffu, Xl.z, 0);
+                const bool mv = G.p >= 0;
+                const int dx = mv ? (int)(Xl.x - X0x) : 0, dy = mv ? (int)(Xl.y - X0y) : 0, dz = mv ? (int)(Xl.z - X0z) : 0;
+                const int lx = warp_min(dx), ly = warp_min(dy), lz = warp_min(dz);
+                const long long sx = (long long)warp_max(dx) - lx, sy = (long long)warp_max(dy) - ly,
+                                sz = (long long)warp_max(dz) - lz;
+                gok = sx < (1ll << 30) && sy < (1ll << 30) && sz < (1ll << 30);
+                Gc = make_uint4(X0x + (unsigned)(lx + (int)(sx >> 1)), X0y + (unsigned)(ly + (int)(sy >> 1)),
+                                X0z + (unsigned)(lz + (int)(sz >> 1)), 0u);
+                const float up = 1.f + 3.814697265625e-06f;   // 2^-18: also the rounding of offsets this size
+                gex = fmaf((float)sx, 0.5f * up, 4.f);
+                gey = fmaf((float)sy, 0.5f * up, 4.f);
+                gez = fmaf((float)sz, 0.5f * up, 4.f);
+            }
+            int nq = 0;   // children waiting
             bool done = sp == 0;
             for (;;) {
                 int ml = 0, mn = 0;
@@ -490,27 +516,66 @@ __global__ void __launch_bounds__(kWppThreads, 5) k_gravity(GravArgs a) {
                     __syncwarp();
                 }
                 if (done) break;
-                // the children of up to four opened nodes, one per lane
-                const int npop = sp <= 96 ? min(4, sp) : 1;
-                const int slot = (int)(lane >> 3);
-                int lev = -1, child = -1;
-                unsigned mask = 0u;
-                if (slot < npop) {
-                    const unsigned en = (unsigned)sm.stk[sp - 1 - slot];
-                    const int k = (int)(en >> 28), c = (int)(en & 0x0fffffffu) * kFan + (int)(lane & 7u);
-                    if (c < B.lvl_n[k - 1]) {
-                        lev = k - 1;
-                        child = c;
-                        mask = sm.stm[sp - 1 - slot];
-                    }
-                }
-                __syncwarp();
-                sp -= npop;
-                const int id = B.lvl_off[max(lev, 0)] + max(child, 0);
+                int lev, child, id;
+                unsigned mask;
                 GravNode N;
-                N.lo = a.node_lo[id];
-                N.hi = a.node_hi[id];
-                grav_node(N, gb.rcu, a.inv_theta);
+                // the children of up to four opened nodes, one per lane
+                auto pop = [&]() {
+                    const int npop = sp <= 96 ? min(4, sp) : 1;
+                    const int slot = (int)(lane >> 3);
+                    lev = child = -1;
+                    mask = 0u;
+                    if (slot < npop) {
+                        const unsigned en = (unsigned)sm.stk[sp - 1 - slot];
+                        const int k = (int)(en >> 28), c = (int)(en & 0x0fffffffu) * kFan + (int)(lane & 7u);
+                        if (c < B.lvl_n[k - 1]) {
+                            lev = k - 1;
+                            child = c;
+                            mask = sm.stm[sp - 1 - slot];
+                        }
+                    }
+                    __syncwarp();
+                    sp -= npop;
+                };
+                auto load = [&]() {
+                    id = B.lvl_off[max(lev, 0)] + max(child, 0);
+                    N.lo = a.node_lo[id];
+                    N.hi = a.node_hi[id];
+                    grav_node(N, gb.rcu, a.inv_theta);
+                };
+                if (M >= 4) {
+                    while (sp > 0 && nq < 32 && (sp <= 96 || nq == 0)) {
+                        pop();
+                        load();
+                        // a member is no farther from the centre than the half extents
+                        const float gx = fmaxf(fabsf((float)(int)(N.cx - Gc.x)) - N.ex - gex, 0.f),
+                                    gy = fmaxf(fabsf((float)(int)(N.cy - Gc.y)) - N.ey - gey, 0.f),
+                                    gz = fmaxf(fabsf((float)(int)(N.cz - Gc.z)) - N.ez - gez, 0.f);
+                        const bool keep = child >= 0 && !(gok && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) > N.out2);
+                        const unsigned bk = __ballot_sync(0xffffffffu, keep);
+                        if (keep) {
+                            const int o = nq + __popc(bk & lt);
+                            sm.qe[o] = (int)(((unsigned)lev << 28) | (unsigned)child);
+                            sm.qm[o] = (unsigned char)mask;
+                        }
+                        nq += __popc(bk);
+                        __syncwarp();
+                    }
+                    const int k = min(nq, 32);
+                    nq -= k;
+                    lev = child = -1;
+                    mask = 0u;
+                    if ((int)lane < k) {
+                        const unsigned en = (unsigned)sm.qe[nq + (int)lane];
+                        lev = (int)(en >> 28);
+                        child = (int)(en & 0x0fffffffu);
+                        mask = sm.qm[nq + (int)lane];
+                    }
+                    __syncwarp();
+                } else {
+                    pop();
+                }
+                load();
                 unsigned om = 0u;   // members that open the child
 #pragma unroll
                 for (int m = 0; m < M; ++m) {
@@ -532,7 +597,7 @@ __global__ void __launch_bounds__(kWppThreads, 5) k_gravity(GravArgs a) {
                     sm.stm[o] = (unsigned char)om;
                 }
                 sp += __popc(bp);
-                done = sp == 0;
+                done = sp == 0 && nq == 0;
                 __syncwarp();
             }
             // per member: fold its lanes' sums, write its outputs
