@@ -1208,10 +1208,14 @@ __global__ void __launch_bounds__(256) k_list_sort(int n, int per, int32_t* __re
             int32_t* seg = ext + (size_t)i * kExtCap;
             more = todo != 0u;
             if (more) fetch();
-            if (cc <= 64) {   // one or two entries per lane: the rank among the cc
+            if (cc <= 32) {   // one entry per lane: its rank among the cc
+                int r0 = 0;
+                for (int k = 0; k < cc; ++k) r0 += __shfl_sync(0xffffffffu, w0, k) < w0;
+                __syncwarp();   // every lane has read the segment before it is overwritten
+                if ((int)lane < cc) seg[r0] = w0;
+            } else if (cc <= 64) {   // two
                 int r0 = 0, r1 = 0;
-                const int c0 = min(cc, 32);
-                for (int k = 0; k < c0; ++k) {
+                for (int k = 0; k < 32; ++k) {
                     const int x = __shfl_sync(0xffffffffu, w0, k);
                     r0 += x < w0;
                     r1 += x < w1;
