@@ -454,10 +454,13 @@ sph_status sph_gravity(sph_ctx *ctx, const sph_grid *grid, const int32_t *active
  * writes dL/dx (g_pos, n x 3), dL/du (g_u, n) and dL/dm (g_mass, n) through
  * the whole chain: the implicit dependence of h on the positions
  * (dh/dx = -(dN/dx)/(dN/dh)), rho and d rho/dh, the grad-h factor Omega, the
- * pressure and viscosity terms. Velocities are constants. The pair sets are
- * recomputed by walking the grid (no neighbour lists are stored). FP32 pair
- * terms with compensated sums; deterministic (gathers, no atomics). The
- * first call on a grid allocates its adjoint workspace (~56 bytes/particle).
+ * pressure and viscosity terms. Velocities are constants. The pair sets come
+ * from the neighbour lists of the last sph_density call on the grid, if it
+ * recorded them for every particle and each position and h is the one they were
+ * made with (checked on the device); otherwise, and for particles whose list
+ * did not fit, from walking the grid. FP32 pair terms with compensated sums;
+ * deterministic (gathers). The first call on a grid allocates its adjoint
+ * workspace (~64 bytes/particle).
  */
 sph_status sph_backward(sph_ctx *ctx, const sph_grid *grid, const float *vel, const float *u,
                         const float *h, const float *rho, const float *omega, const float *g_acc,

@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* _
 // another in shared memory, ranked and placed as k_rs_pass does. A set this small
 // is one or two tiles of the passes above, and pays their launches and round trips
 // through global memory (about 8 us each) for a microsecond or two of work:
-// 4,096 keys 70 -> 34 us.
+// 4,096 keys 63 -> 34 us.
 constexpr int kRsSmallT = 1024, kRsSmallWarps = kRsSmallT / 32;
 static_assert(kRsSmall == kRsSmallT * kRsIPT, "items of the block");
 struct RsSmallSmem {
