@@ -749,8 +749,13 @@ cudaError_t launch_force_wpp(sph_ctx* ctx, const ForceLaunch& a, int64_t n_activ
         c.list_st = g->list_st;
         c.list_ep = g->list_ep;
         c.fb_list = g->fb_list;
-        const int lb = (int)std::max<long long>(
-            1, std::min<long long>((long long)ctx->sm_count * 16, (n_active + 4 * kFlPer - 1) / (4 * kFlPer)));
+        // Blocks of a few steps per warp: lists differ in length by a factor of ten and
+        // more, and the block scheduler evens that out (16 blocks per SM, a share of the
+        // set each, left a fifth of the SMs' time idle at the end). At least 30 per SM,
+        // else seven steps per warp: conduction of 800k 0.84 -> 0.77 ms, 2M force call
+        // 1.40 -> 1.23; a queue in their place cost more than it gave.
+        const long long all = (n_active + 4 * kFlPer - 1) / (4 * kFlPer);
+        const int lb = (int)std::max<long long>(1, std::min(all, std::max<long long>(ctx->sm_count * 30ll, all / 7)));
         launch_force_list(a.hash != nullptr, visc, c.fcond != nullptr, lb, s, c);
         ++ctx->launches;
         c.fb_act = g->fb_list;
