@@ -317,29 +317,34 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_density_mp(WppArgs a) {
                     double HH = -1.0;
                     const bool self = run && sub == 0;   // the self term: w(0) = 1, q w'(0) = 0
                     // Two entries per lane per step (k and k + 4), their terms in packed
-                    // arithmetic. An entry outside h counts as one far beyond it (w = w' = 0),
-                    // a coincident one as one at the smallest normal distance (w = 1, w' = 0).
+                    // arithmetic. An entry outside h, or past the list's end, takes q = 2
+                    // (w = w' = 0) whatever its distance: no squared distance is beyond every h.
+                    // (Below the smallest normal r^2 the root is that one's: w = 1, w' = 0.)
                     // The sums of w and q w', which fix h to the last bit, are added one
                     // entry at a time. (10M 100 % call: -1.5 % against scalar terms.)
                     float Sw = self ? 1.f : 0.f, Sdw = 0.f;
                     float2 MW = make_float2(self ? __uint_as_float(Xm.w) : 0.f, 0.f), MQ = both(0.f);
                     int nn = 0;
                     const int kend = run ? cm : 0;
-                    auto take = [&](int k) {
-                        float2 e = k < kend ? mp.d[mm][k] : make_float2(1e30f, 0.f);
-                        bool in = e.x < lo2;
+                    auto take = [&](int k, bool& in) {
+                        // (past the end: beyond every bound, so that nothing there is read)
+                        const float2 e = k < kend ? mp.d[mm][k] : make_float2(INFINITY, 0.f);
+                        in = e.x < lo2;
                         if (!in && e.x < hi2) {   // the thin band: the exact predicate
                             if (HH < 0.0) HH = wpp_hh(h, B);
                             in = exact_pred(exact_d2(Xm, a.posm[jm[k]]), HH);
                         }
                         nn += in ? 1 : 0;
-                        e.x = in ? fmaxf(e.x, 1.1754944e-38f) : 1e30f;
                         return e;
                     };
                     for (int k = sub; __any_sync(0xffffffffu, k < kend); k += 8) {
-                        const float2 e0 = take(k), e1 = take(k + 4);
+                        bool in0, in1;
+                        const float2 e0 = take(k, in0), e1 = take(k + 4, in1);
                         const float2 r2 = make_float2(e0.x, e1.x), m = make_float2(e0.y, e1.y);
-                        const float2 q = mul2(mul2(r2, make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y))), both(hinv));
+                        const float2 rinv = make_float2(rsqrt_ftz(fmaxf(r2.x, FLT_MIN)), rsqrt_ftz(fmaxf(r2.y, FLT_MIN)));
+                        float2 q = mul2(mul2(r2, rinv), both(hinv));
+                        q.x = in0 ? q.x : 2.f;
+                        q.y = in1 ? q.y : 2.f;
                         float2 w, dw;
                         spline_pair(q, w, dw);
                         const float2 qdw = mul2(q, dw);
