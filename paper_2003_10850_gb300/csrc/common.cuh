@@ -140,7 +140,8 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
     return y;
 }
 
-// 1/x without the denormal cases, as __fdividef takes it
+// 1/x, a subnormal x taken as zero (callers keep x normal) and a subnormal result as
+// zero (__fdividef does the second, not the first)
 __device__ __forceinline__ float rcp_ftz(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -675,6 +675,7 @@ struct WppForceI {
     float f;                       // Balsara factor (1 without the switch)
     float u, kap;                  // conduction: u and conductivity (unused without it)
     float al;                      // own viscosity parameter (VISC = 2 only)
+    float rhoinv;                  // 1/rho (packed form with conduction only)
 };
 
 // Viscosity variants of the force pair term: kViscScalar, one alpha for every
@@ -737,6 +738,10 @@ struct WppForceS2 {
 // largest part of what the list passes issue between their gathers. d = x_j - x_i, v = (v_j, m_j), th =
 // (rho_j, A_j, c_j, 1/h_j), b and c as wpp_force_pair; two false: the second
 // pair is none. A coincident pair adds its sound speeds to v_sig and no force.
+// The reciprocals take a subnormal divisor as zero, so none is formed of a value
+// that may be one: m_j/(rho_i rho_j) takes two factors in place of the product (for
+// rho_i + rho_j to be subnormal rho^2 has underflowed, and A is no number already),
+// and conductivities whose sum is subnormal conduct nothing (4 k_i k_j is zero).
 template <int VISC, bool COND>
 __device__ __forceinline__ void wpp_force_pair2(const WppForceI& I, float2 dx, float2 dy, float2 dz, float4 v0, float4 v1,
                                                 float4 th0, float4 th1, float2 b0, float2 b1, float2 c0, float2 c1,
@@ -768,9 +773,9 @@ __device__ __forceinline__ void wpp_force_pair2(const WppForceI& I, float2 dx, f
     if (COND) {
         const float2 kj = make_float2(c0.y, c1.y), ks = add2(both(I.kap), kj);
         float2 kij = mul2(mul2(both(4.f * I.kap), kj), rcp2_ftz(ks));
-        kij.x = ks.x > 0.f ? kij.x : 0.f;
-        kij.y = ks.y > 0.f ? kij.y : 0.f;
-        const float2 mr = mul2(m, rcp2_ftz(mul2(both(I.rho), rj)));
+        kij.x = ks.x >= FLT_MIN ? kij.x : 0.f;
+        kij.y = ks.y >= FLT_MIN ? kij.y : 0.f;
+        const float2 mr = mul2(mul2(m, both(I.rhoinv)), rcp2_ftz(rj));
         S.c = fma2(mul2(mul2(mr, kij), sub2(both(I.u), make_float2(c0.x, c1.x))), Fbar, S.c);
     }
     const float2 PF = mul2(PI, Fbar);

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(128, COND ? 5 : 6) k_force_list(WppArgs a) {
         const float2 ci = COND ? a.fcond[pp] : make_float2(0.f, 0.f);
         const float2 bi = wpp_visc_i<VISC>(a, pp);
         const WppForceI I = {vi.x, vi.y, vi.z, thi.w, thi.x, thi.y, thi.z, kNorm * thi.w * thi.w * thi.w * thi.w,
-                             bi.x, ci.x, ci.y, bi.y};
+                             bi.x, ci.x, ci.y, bi.y, COND ? 1.f / thi.x : 0.f};
         WppForceS2 S;
         unsigned long long hs = 0;
         const int tot = live ? cn + (int)ec : 0;
@@ -577,7 +577,8 @@ __global__ void __launch_bounds__(kWppThreads, MINB) k_force_mp(WppArgs a) {
                     const float2 ci = COND ? a.fcond[p] : make_float2(0.f, 0.f);
                     const float2 bi = wpp_visc_i<VISC>(a, p);
                     const WppForceI I = {vi.x, vi.y, vi.z, thi.w, thi.x, thi.y, thi.z,
-                                         kNorm * thi.w * thi.w * thi.w * thi.w, bi.x, ci.x, ci.y, bi.y};
+                                         kNorm * thi.w * thi.w * thi.w * thi.w, bi.x, ci.x, ci.y, bi.y,
+                                         COND ? 1.f / thi.x : 0.f};
                     WppForceS2 S;
                     unsigned long long hs = 0;
                     const int32_t* lst = pj + mq * kFmCap;

@@ -2,9 +2,11 @@
 whose intermediate values leave the normal numbers or pass any fixed constant."""
 import numpy as np
 import pytest
+import torch
 
+import oracle
 import workloads as W
-from sph_cases import as_f32, gpu_density, gpu_grid
+from sph_cases import as_f32, check_force, dev, gpu_density, gpu_grid, host, oracle_all
 
 pytestmark = pytest.mark.gpu
 
@@ -40,3 +42,44 @@ def test_density_scales_with_the_box(S, ctx, exp):
     assert np.array_equal(g2["h"].astype(np.float64), g1["h"].astype(np.float64) * f)
     for k in ("n_ngb", "hash", "omega"):
         assert np.array_equal(g1[k], g2[k]), k
+
+
+@pytest.fixture(scope="module")
+def lattice():
+    p = as_f32(W.config1(16))
+    return p, oracle_all(p)
+
+
+# masses and densities times 2^-66: rho_i rho_j is subnormal; kappa times 2^-130:
+# kappa_i + kappa_j is
+@pytest.mark.parametrize("mexp,kexp", [(-66, 0), (0, -130)])
+@pytest.mark.parametrize("lists", [True, False])
+def test_conduction_with_subnormal_divisors(S, ctx, lattice, mexp, kexp, lists):
+    """From the recorded lists and walked, within the force tests' tolerances; a
+    conductivity whose products underflow conducts nothing."""
+    p, (X, d, _) = lattice
+    h, rho, om = (d[k].astype(np.float32) for k in ("h", "rho", "omega"))
+    fm, fk = np.float32(2.0 ** mexp), np.float32(2.0 ** kexp)
+    kappa = np.random.default_rng(11).uniform(0.1, 2.0, p.n).astype(np.float32) * fk
+    q = W.Particles(p.pos, p.vel, p.mass * float(fm), p.u, p.box)
+    rq = rho * fm
+    f = oracle.force(X, p.vel, q.mass, p.u, h, rq, om)
+    co, cs = oracle.conduction(X, q.mass, p.u, h, rq, kappa)
+    grid = gpu_grid(S, ctx, q, S.default_params())
+    if lists:
+        S.density(ctx, grid, dev(h), None, S.default_params(flags=S.SPH_FIXED_H))
+    n = p.n
+    acc, du, vs = torch.zeros(n, 3, device="cuda"), torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
+    dc = torch.zeros(n, device="cuda")
+    hs = torch.zeros(n, dtype=torch.int64, device="cuda")
+    S.sph_hydro_force_conduction(ctx, grid, dev(p.vel), dev(p.u), dev(h), dev(rq), dev(om), None, None, dev(kappa),
+                                 None, acc, du, vs, dc, hs, S.default_params())
+    rc, st = S.sph_sync_status(ctx, raise_on_error=False)
+    assert rc == 0 and (st["list_force"] == n) == lists
+    check_force({"acc": host(acc), "dudt": host(du), "vsig": host(vs), "hash": host(hs).view(np.uint64)}, f,
+                np.arange(n), 1e-4)
+    dcg = host(dc).astype(np.float64)
+    if kexp:   # 4 kappa_i kappa_j underflows
+        assert np.all(dcg == 0.0)
+    else:
+        assert np.all(np.abs(dcg - co) <= 1e-4 * cs)
