@@ -191,8 +191,7 @@ __global__ void k_grav_box_rc(const BoxDesc* __restrict__ boxes, int nb, double 
     gb[b] = g;
 }
 
-// Approximations without the denormal cases (none occur: r^3 stays far inside
-// the normal range and an exponential that small adds nothing).
+// 2^x, a subnormal result as zero (an exponential that small adds nothing).
 __device__ __forceinline__ float grav_ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -211,8 +210,10 @@ __device__ __forceinline__ float grav_soft(float q) {
 // erfc from Abramowitz & Stegun 7.1.26 (Hastings' rational approximation,
 // |error| <= 1.5e-7): erfc(x) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) e^{-x^2},
 // t = 1 / (1 + p x), so that both terms share one exponential.
+// 1/r^3 goes in as 1/r^2, then 1/r: r^3 is subnormal for pairs closer than 2.3e-13
+// (box units; any box smaller than 1e-3 has some), where the softened term is not.
 __device__ __forceinline__ float2 grav_K(const GravArgs& a, float2 r2) {
-    const float2 r = mul2(r2, make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)));
+    const float2 rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)), r = mul2(r2, rinv);
     float2 K = both(1.f);
     if (r.x < a.hs) K.x = grav_soft(r.x * a.inv_hs);
     if (r.y < a.hs) K.y = grav_soft(r.y * a.inv_hs);
@@ -228,8 +229,7 @@ __device__ __forceinline__ float2 grav_K(const GravArgs& a, float2 r2) {
         const float2 z = mul2(mul2(x, x), both(-1.4426950409f));   // log2 e
         K = mul2(K, mul2(make_float2(grav_ex2(z.x), grav_ex2(z.y)), e));
     }
-    const float2 r3 = mul2(r2, r);
-    return mul2(K, make_float2(rcp_ftz(r3.x), rcp_ftz(r3.y)));
+    return mul2(mul2(K, rcp2_ftz(r2)), rinv);
 }
 
 // One axis of the exact coarse box geometry: squared gap, squared far-side

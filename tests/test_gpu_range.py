@@ -83,3 +83,29 @@ def test_conduction_with_subnormal_divisors(S, ctx, lattice, mexp, kexp, lists):
         assert np.all(dcg == 0.0)
     else:
         assert np.all(np.abs(dcg - co) <= 1e-4 * cs)
+
+
+# pairs 3 to 12 integer units apart inside the softening, and 11 to 15 units without
+# one: r^3 is subnormal (r below 2.3e-13), the term is not
+@pytest.mark.parametrize("soft,units", [(0.01, (3, 5, 8, 12)), (0.0, (11, 12, 13, 15))])
+def test_gravity_of_close_pairs_in_a_small_box(S, ctx, soft, units):
+    """Counts exact, accelerations within the gravity tests' 2e-5 of the
+    per-particle scale."""
+    L = 2.0 ** -14
+    rng = np.random.default_rng(19)
+    n = 512
+    pos = np.rint(rng.random((n, 3)) * 2.0 ** 32) * (L * 2.0 ** -32)
+    mate = pos[: n // 2].copy()
+    mate[:, 0] += np.resize(np.array(units), n // 2) * (L * 2.0 ** -32)
+    pos = np.concatenate([pos, mate]) % L
+    mass = rng.uniform(0.5, 1.5, len(pos)).astype(np.float32).astype(np.float64) / len(pos)
+    sp = dict(theta=0.5, r_split=0.05 * L, r_cut=0.2 * L, h_soft=soft * L)
+    o = oracle.gravity(oracle.quantize(pos, L), mass, box=L, **sp)
+    grid = S.sph_build_grid(ctx, dev(pos, torch.float64), dev(mass), S.default_params(box=L))
+    acc = torch.zeros(len(pos), 3, device="cuda")
+    nn, npr = (torch.zeros(len(pos), dtype=torch.int32, device="cuda") for _ in range(2))
+    S.sph_gravity(ctx, grid, None, S.gravity_params(**sp), acc, nn, npr)
+    S.sph_sync_status(ctx)
+    assert np.array_equal(host(nn), o["n_nodes"]) and np.array_equal(host(npr), o["n_pairs"])
+    err = np.linalg.norm(host(acc) - o["acc"], axis=1)
+    assert np.all(err <= 2e-5 * o["scale"]), (err / o["scale"]).max()
