@@ -93,7 +93,9 @@ __global__ void k_quantize(const P* __restrict__ pos, const float* __restrict__ 
 // the digit totals and from the tiles before it, whose counts it reads as they
 // appear (each tile publishes its own counts first, then its running totals).
 // Tiles are numbered by a ticket, so a tile only ever waits for tiles that
-// already run. 63-bit keys take 7 passes of 9 bits: 9 launches in all.
+// already run; a wait is bounded, and a tile whose wait runs out counts the items
+// before it by itself, so that the result never depends on the wait. 63-bit keys
+// take 7 passes of 9 bits: 9 launches in all.
 //
 // What bounds it: at 10M keys the 24 bytes per item and pass (HBM); below a
 // few hundred thousand the chain of passes, a few microseconds each. A
@@ -103,7 +105,10 @@ __global__ void k_quantize(const P* __restrict__ pos, const float* __restrict__ 
 constexpr int kRsT = 512, kRsIPT = 8, kRsWarps = kRsT / 32;
 constexpr int kRsDig = 1 << kRsBits;
 static_assert(kRsTile == kRsT * kRsIPT && kRsDig == kRsT, "one digit per thread");
-constexpr int kRsSpin = 1 << 22;   // polls of a predecessor's word before giving up
+#ifndef SPH_WAIT_POLLS
+#define SPH_WAIT_POLLS (1 << 22)
+#endif
+constexpr int kRsSpin = SPH_WAIT_POLLS;   // polls of a predecessor's word before counting its tile's items
 constexpr int kRsBack = 8;         // predecessors read at a time
 
 struct RsSmem {
@@ -160,14 +165,13 @@ __device__ __forceinline__ unsigned long long rs_get(const unsigned long long* p
 // digits in lane order, then round order: stable), the block adds the warps
 // before, and the items leave through shared memory in digit order, so that
 // consecutive threads write consecutive places of a digit's run. vin NULL: the
-// items' own indices. ctr (may be NULL) receives ST_TIMEOUT if a wait ran out;
-// every store stays inside [0, n) in any case.
+// items' own indices.
 __global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* __restrict__ kin,
                                                      const unsigned* __restrict__ vin,
                                                      unsigned long long* __restrict__ kout,
                                                      unsigned* __restrict__ vout, int n, int pass,
                                                      const unsigned* __restrict__ hist, unsigned* ticket,
-                                                     unsigned long long* status, Counters* ctr) {
+                                                     unsigned long long* status) {
     extern __shared__ __align__(16) unsigned char raw[];
     RsSmem& sm = *reinterpret_cast<RsSmem*>(raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -275,12 +279,17 @@ __global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* _
                 if (tag == incl) more = false;
             }
         }
-        if (t >= 0 && !more && ++spins > kRsSpin) {
-            if (ctr) atomicOr(&ctr->status, ST_TIMEOUT);
-            break;
-        }
+        if (t >= 0 && !more && ++spins > kRsSpin) break;
     }
-    if (tile > 0 && t < 0) rs_put(mine, incl, prefix + cnt);
+    if (__syncthreads_or(t >= 0)) {   // a wait ran out: count the items before the tile (nobody writes kin)
+        sm.gbase[tid] = 0u;
+        __syncthreads();
+        for (long long i = tid; i < base; i += kRsT)
+            atomicAdd(&sm.gbase[(unsigned)(kin[i] >> shift) & (kRsDig - 1u)], 1u);
+        __syncthreads();
+        prefix = sm.gbase[tid];
+    }
+    if (tile > 0) rs_put(mine, incl, prefix + cnt);
     sm.gbase[tid] = (unsigned)(x >> 32) + prefix - sm.start[tid];
     __syncthreads();
 #pragma unroll
@@ -289,7 +298,7 @@ __global__ void __launch_bounds__(kRsT, 2) k_rs_pass(const unsigned long long* _
         if (p < tn) {
             const unsigned long long k = sm.key[p];
             const unsigned g = sm.gbase[(unsigned)(k >> shift) & (kRsDig - 1u)] + (unsigned)p;
-            if (g < (unsigned)n) {
+            if (g < (unsigned)n) {   // (always, unless the caller's keys change under the sort)
                 kout[g] = k;
                 vout[g] = sm.val[p];
             }
@@ -419,8 +428,8 @@ __global__ void __launch_bounds__(kRsSmallT) k_rs_small(const unsigned long long
 // kin may be kb, with an even number kin may not be ka. (Up to kRsSmall items go
 // straight to where the last pass would end.)
 cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsigned* va, unsigned long long* kb,
-                    unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, Counters* ctr,
-                    cudaStream_t s, unsigned* launches) {
+                    unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, cudaStream_t s,
+                    unsigned* launches) {
     const int passes = (key_bits + kRsBits - 1) / kRsBits;
     const int tiles = (n + kRsTile - 1) / kRsTile;
     if (n <= kRsSmall) {
@@ -442,8 +451,7 @@ cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsig
     for (int p = 0; p < passes; ++p) {
         k_rs_pass<<<tiles, kRsT, sizeof(RsSmem), s>>>(p == 0 ? kin : p & 1 ? ka : kb,
                                                       p == 0 ? nullptr : p & 1 ? va : vb, p & 1 ? kb : ka,
-                                                      p & 1 ? vb : va, n, p, hist + p * kRsDig, ticket + p, status,
-                                                      ctr);
+                                                      p & 1 ? vb : va, n, p, hist + p * kRsDig, ticket + p, status);
         if ((e = cudaGetLastError())) return e;
     }
     *launches += 1 + passes;
@@ -454,12 +462,11 @@ cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsig
 // a3: gather into sorted order, hierarchy bounding boxes, h_max
 // ---------------------------------------------------------------------------
 
-__global__ void k_gather(const uint4* __restrict__ xq, int n, uint4* __restrict__ posm, int32_t* __restrict__ perm,
+__global__ void k_gather(const uint4* __restrict__ xq, int n, uint4* __restrict__ posm, const int32_t* __restrict__ perm,
                          int32_t* __restrict__ rank) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     int i = perm[k];
-    if ((unsigned)i >= (unsigned)n) perm[k] = i = k;   // only after a sort whose wait ran out (ST_TIMEOUT)
     posm[k] = xq[i];
     rank[i] = k;
 }
@@ -653,16 +660,17 @@ __global__ void k_mark(const int32_t* __restrict__ active, int na, const int32_t
 
 // The indices whose flag is set, ascending, and their number, in one pass:
 // a tile of 4096 flags counts its own, publishes the count, and adds the counts
-// of the tiles before it (as k_rs_pass; 32 of them at a time). flag: a byte per
-// index, or (max_bin >= 0) its time bin, set if the bin ends a step at `tick`.
-// work: a ticket and a word per tile, cleared. One launch in place of a
-// three-launch scan and a placing pass over every flag and its scan.
+// of the tiles before it (32 of them at a time), or counts their flags itself when
+// a wait runs out (as k_rs_pass). flag: a byte per index, or (max_bin >= 0) its time
+// bin, set if the bin ends a step at `tick`. work: a ticket and a word per tile,
+// cleared. One launch in place of a three-launch scan and a placing pass over every
+// flag and its scan.
 constexpr int kCpT = 256, kCpPer = 16;
 static_assert(kCpTile == kCpT * kCpPer, "flags per block");
 __global__ void __launch_bounds__(kCpT) k_flag_list(const uint8_t* __restrict__ flag, int n, long long tick, int max_bin,
                                                     unsigned long long* work, int32_t* __restrict__ list,
-                                                    uint32_t* __restrict__ count, Counters* ctr, CallBegin b) {
-    __shared__ unsigned s_tile, s_before, s_warp[kCpT / 32];
+                                                    uint32_t* __restrict__ count, CallBegin b) {
+    __shared__ unsigned s_tile, s_before, s_late, s_warp[kCpT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (blockIdx.x == 0) call_begin(b, tid);
     if (tid == 0) s_tile = atomicAdd(reinterpret_cast<unsigned*>(work), 1u);
@@ -671,13 +679,10 @@ __global__ void __launch_bounds__(kCpT) k_flag_list(const uint8_t* __restrict__ 
     unsigned long long* status = work + 1;
     const long long i0 = (long long)tile * kCpTile + tid * kCpPer;
     unsigned set = 0u;   // bit k: flag i0 + k
-    auto take = [&](int k, unsigned v) {
-        if (max_bin >= 0) {
-            const int b = min((int)v, max_bin);
-            v = (tick & ((1ll << (max_bin - b)) - 1)) == 0 ? 1u : 0u;
-        }
-        set |= v ? 1u << k : 0u;
+    auto is_set = [&](unsigned v) {
+        return max_bin >= 0 ? (tick & ((1ll << (max_bin - min((int)v, max_bin))) - 1)) == 0 : v != 0u;
     };
+    auto take = [&](int k, unsigned v) { set |= is_set(v) ? 1u << k : 0u; };
     if (i0 + kCpPer <= n && (reinterpret_cast<uintptr_t>(flag) & 15) == 0) {
         const uint4 v = *reinterpret_cast<const uint4*>(flag + i0);
         const unsigned w[4] = {v.x, v.y, v.z, v.w};
@@ -702,8 +707,12 @@ __global__ void __launch_bounds__(kCpT) k_flag_list(const uint8_t* __restrict__ 
         before += w < warp ? s_warp[w] : 0u;
         total += s_warp[w];
     }
+    constexpr unsigned kAgg = 1u, kIncl = 2u;
+    auto publish = [&](unsigned prefix) {
+        if (tile > 0) rs_put(status + tile, kIncl, prefix + total);
+        if ((long long)(tile + 1) * kCpTile >= n) *count = min(prefix + total, (unsigned)n);
+    };
     if (warp == 0) {
-        constexpr unsigned kAgg = 1u, kIncl = 2u;
         if (lane == 0) rs_put(status + tile, tile == 0 ? kIncl : kAgg, total);
         unsigned prefix = 0u;
         int t = tile - 1;
@@ -716,18 +725,23 @@ __global__ void __launch_bounds__(kCpT) k_flag_list(const uint8_t* __restrict__ 
             const int use = fi < fw ? fi + 1 : fw;   // words that count: up to the first running total
             prefix += warp_sum(lane < use ? (unsigned)w : 0u);
             t = fi < fw ? -1 : t - fw;
-            if (fw < fi && ++spins > kRsSpin) {
-                if (lane == 0 && ctr) atomicOr(&ctr->status, ST_TIMEOUT);
-                break;
-            }
+            if (fw < fi && ++spins > kRsSpin) break;
         }
         if (lane == 0) {
-            if (tile > 0 && t < 0) rs_put(status + tile, kIncl, prefix + total);
-            s_before = prefix;
-            if ((long long)(tile + 1) * kCpTile >= n) *count = min(prefix + total, (unsigned)n);
+            s_late = t >= 0 ? 1u : 0u;
+            s_before = t >= 0 ? 0u : prefix;
+            if (t < 0) publish(prefix);
         }
     }
     __syncthreads();
+    if (s_late) {   // a wait ran out: count the flags before the tile
+        unsigned k = 0u;
+        for (long long i = tid; i < (long long)tile * kCpTile; i += kCpT) k += is_set(flag[i]) ? 1u : 0u;
+        k = warp_sum(k);
+        if (lane == 0) atomicAdd(&s_before, k);
+        __syncthreads();
+        if (tid == 0) publish(s_before);
+    }
     unsigned pos = s_before + before;
     while (set) {
         const int k = __ffs(set) - 1;
@@ -787,8 +801,8 @@ static cudaError_t grid_fill(sph_grid* g, const void* pos, int f64, const float*
                                                  g->xq, g->k2, ctx->counters);
     ++ctx->launches;
     static_assert(((63 + kRsBits - 1) / kRsBits) % 2 == 1, "an odd number of passes ends in (keys, perm)");
-    const cudaError_t e = rs_sort(g->k2, keys, (unsigned*)g->perm, g->k2, g->v2, n, 63, g->rs_work, ctx->sm_count,
-                                  ctx->counters, s, &ctx->launches);
+    const cudaError_t e =
+        rs_sort(g->k2, keys, (unsigned*)g->perm, g->k2, g->v2, n, 63, g->rs_work, ctx->sm_count, s, &ctx->launches);
     if (e) return e;
     k_gather<<<blocks, 256, 0, s>>>(g->xq, n, g->posm, g->perm, g->rank);
     k_tree_low<<<dim3((g->max_leaves + kTreeT - 1) / kTreeT, nb), kTreeT, 0, s>>>(
@@ -933,7 +947,7 @@ void flag_list(sph_grid* g, const uint8_t* flag, long long tick, int max_bin, in
     const int n = (int)g->n;
     k_flag_list<<<(n + kCpTile - 1) / kCpTile, kCpT, 0, s>>>(flag, n, tick, max_bin,
                                                              (unsigned long long*)(g->flag + flag_bytes(n)), list, count,
-                                                             g->ctx->counters, b);
+                                                             b);
     ++g->ctx->launches;
 }
 

@@ -176,8 +176,8 @@ constexpr size_t rs_work_bytes(int64_t n) {
     return kRsHead + sizeof(unsigned long long) * (1 << kRsBits) * (size_t)((n + kRsTile - 1) / kRsTile);
 }
 cudaError_t rs_sort(const unsigned long long* kin, unsigned long long* ka, unsigned* va, unsigned long long* kb,
-                    unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, Counters* ctr,
-                    cudaStream_t s, unsigned* launches);
+                    unsigned* vb, int n, int key_bits, unsigned char* work, int sm_count, cudaStream_t s,
+                    unsigned* launches);
 // SPH_TIME_KERNELS support: event pair around one kernel launch
 cudaEvent_t timing_event(sph_ctx* ctx);
 

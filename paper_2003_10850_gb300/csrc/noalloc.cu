@@ -71,7 +71,7 @@ extern "C" sph_status sph_sort_keys_static(const uint64_t* keys, int64_t n, uint
         return SPH_ERR_CUDA;
     if (sph::rs_sort(reinterpret_cast<const unsigned long long*>(keys), kb, vb,
                      reinterpret_cast<unsigned long long*>(sorted_keys), reinterpret_cast<unsigned*>(perm), nn, 64,
-                     base + kOffWork, sms, nullptr, s, &launches) != cudaSuccess)
+                     base + kOffWork, sms, s, &launches) != cudaSuccess)
         return SPH_ERR_CUDA;
     return SPH_OK;
 }
