@@ -11,6 +11,11 @@
 //    whose list overflows works it off as it fills, once per iteration.
 //  - force: each particle's A, c, 1/h and predicate bound are formed once per
 //    call (k_f64_pack), not once per pair.
+// Sums: at most eight terms of a lane plainly, everything above that (further terms,
+// the lanes) with the rounding errors carried along, in the density pass once per
+// particle. It is 5 % of the two passes' time; errors in units of 2^-53 of the sum of
+// the magnitudes (55 to 100 pairs, simulated): 0.4, with a plain fold 0.8, with Kahan's
+// sum over plain sums of leaves 0.6.
 // One particle per thread, every candidate tested and every square root and
 // division taken in FP64 in the pair loop, took 2.9 + 3.1 ms (density + force)
 // for 32,768 lattice particles; this form takes 0.71 + 0.54 ms.
@@ -30,19 +35,67 @@ struct F64Smem {
 };
 static_assert(kWppWarps * sizeof(F64Smem) <= 48 * 1024, "static shared memory");
 
-// Sums of four per-lane values over the warp, in every lane.
+// a + b rounded, with the rounding error in e: the larger exponent first (compared as
+// integers), then three FP64 additions.
+__device__ __forceinline__ double f64_two_sum(double a, double b, double& e) {
+    const bool sw = (__double2hiint(a) & 0x7fffffff) < (__double2hiint(b) & 0x7fffffff);
+    const double l = sw ? b : a, r = sw ? a : b, t = __dadd_rn(l, r);
+    e = __dsub_rn(r, __dsub_rn(t, l));
+    return t;
+}
+
+// Sums of two per-lane values over the warp, in every lane.
+__device__ __forceinline__ void f64_fold2(double& x, double& y) {
+    const bool lo16 = lane_id() < 16u;
+    double s = (lo16 ? x : y) + __shfl_xor_sync(0xffffffffu, lo16 ? y : x, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    x = __shfl_sync(0xffffffffu, s, 0);
+    y = __shfl_sync(0xffffffffu, s, 16);
+}
+
+// Sums of four per-lane values over the warp, in every lane, the additions' errors
+// carried along and added at the end: four times the additions of a plain fold, so the
+// density kernel takes it once per particle, not once per evaluation.
 __device__ __forceinline__ void f64_fold4(double& x, double& y, double& z, double& u) {
     const bool lo16 = lane_id() < 16u, lo8 = (lane_id() & 8u) == 0u;
-    const double a = (lo16 ? x : z) + __shfl_xor_sync(0xffffffffu, lo16 ? z : x, 16);
-    const double b = (lo16 ? y : u) + __shfl_xor_sync(0xffffffffu, lo16 ? u : y, 16);
-    double s = (lo8 ? a : b) + __shfl_xor_sync(0xffffffffu, lo8 ? b : a, 8);
+    double ea, eb, e;
+    const double a = f64_two_sum(lo16 ? x : z, __shfl_xor_sync(0xffffffffu, lo16 ? z : x, 16), ea);
+    const double b = f64_two_sum(lo16 ? y : u, __shfl_xor_sync(0xffffffffu, lo16 ? u : y, 16), eb);
+    double s = f64_two_sum(lo8 ? a : b, __shfl_xor_sync(0xffffffffu, lo8 ? b : a, 8), e);
+    double c = __dadd_rn(__dadd_rn(lo8 ? ea : eb, __shfl_xor_sync(0xffffffffu, lo8 ? eb : ea, 8)), e);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    for (int o = 4; o > 0; o >>= 1) {
+        const double c2 = __shfl_xor_sync(0xffffffffu, c, o);
+        s = f64_two_sum(s, __shfl_xor_sync(0xffffffffu, s, o), e);
+        c = __dadd_rn(__dadd_rn(c, c2), e);
+    }
+    s = __dadd_rn(s, c);
     x = __shfl_sync(0xffffffffu, s, 0);
     y = __shfl_sync(0xffffffffu, s, 8);
     z = __shfl_sync(0xffffffffu, s, 16);
     u = __shfl_sync(0xffffffffu, s, 24);
 }
+
+// Four per-lane sums, taken up part by part: a part of a few terms is a plain sum (as
+// a leaf's is on the other paths), the parts are added with Kahan's compensation.
+struct F64Sum4 {
+    double x = 0.0, y = 0.0, z = 0.0, u = 0.0, cx = 0.0, cy = 0.0, cz = 0.0, cu = 0.0;
+    __device__ __forceinline__ void add(double& px, double& py, double& pz, double& pu) {
+        kahan_add(x, cx, px);
+        kahan_add(y, cy, py);
+        kahan_add(z, cz, pz);
+        kahan_add(u, cu, pu);
+        px = py = pz = pu = 0.0;
+    }
+    __device__ __forceinline__ void fold(double& px, double& py, double& pz, double& pu) const {
+        px = x; py = y; pz = z; pu = u;
+        double dx = cx, dy = cy, dz = cz, du = cu;
+        f64_fold4(px, py, pz, pu);
+        f64_fold4(dx, dy, dz, du);
+        px -= dx; py -= dy; pz -= dz; pu -= du;
+    }
+};
 
 // The candidates of the walk's leaf list, 32 per step: cand(q, X, valid).
 template <class Cand>
@@ -88,7 +141,8 @@ __global__ void __launch_bounds__(kWppThreads) k_density_f64(WppArgs a) {
         unsigned st = 0;
         bool direct = false;   // the list overflowed: every evaluation sweeps again
         int nnear = 0;
-        double Sw, Sdw, Smw, Smdw;
+        double Sw, Sdw, Smw, Smdw;   // per-lane sums: at most five terms of a list
+        F64Sum4 Q;                   // of the lists already worked off (direct)
         int nn;
         unsigned long long hs;
         // distances of the list's entries
@@ -131,6 +185,7 @@ __global__ void __launch_bounds__(kWppThreads) k_density_f64(WppArgs a) {
                         if (direct) {
                             prepare();
                             accumulate(hinv, HH);
+                            Q.add(Sw, Sdw, Smw, Smdw);
                             __syncwarp();
                             nnear = 0;
                         } else {
@@ -167,20 +222,29 @@ __global__ void __launch_bounds__(kWppThreads) k_density_f64(WppArgs a) {
                 Rw = a.fixed_h ? h : h * a.walk_r;
                 direct = !sweep(Rw, hinv, HH);
             }
-            if (direct) sweep(h, hinv, HH);
+            if (direct) {
+                Q = F64Sum4();
+                sweep(h, hinv, HH);
+            }
             accumulate(hinv, HH);
             __syncwarp();
-            f64_fold4(Sw, Sdw, Smw, Smdw);
+            if (direct) Q.add(Sw, Sdw, Smw, Smdw);
+            // what moves h takes a plain fold: its rounding, below 2^-49 of N, is 2^-27 of
+            // what the smallest step of h (FP32) changes; the outputs' sums are folded below
+            double fw = direct ? Q.x - Q.cx : Sw, fdw = direct ? Q.y - Q.cy : Sdw;
+            f64_fold2(fw, fdw);
             ++c_evals;
-            const double f = (32.0 / 3.0) * Sw - a.n_target;
+            const double f = (32.0 / 3.0) * fw - a.n_target;
             if (a.fixed_h || fabs(f) <= a.n_tol) break;
             if (it >= a.max_iter) {
                 st |= ST_NOT_CONVERGED;
                 break;
             }
-            const float N = (float)((32.0 / 3.0) * Sw), dN = -(32.f / 3.f) * (float)Sdw / h;
+            const float N = (float)((32.0 / 3.0) * fw), dN = -(32.f / 3.f) * (float)fdw / h;
             if (!h_update(h, f, N, dN, (float)a.n_target, cap, blo, bhi, dold, st)) break;
         }
+        if (direct) Q.fold(Sw, Sdw, Smw, Smdw);
+        else f64_fold4(Sw, Sdw, Smw, Smdw);
         nn = warp_sum(nn);
         if (HASH) hs = warp_sum(hs);
         if (lane == 0) {
@@ -239,8 +303,9 @@ __global__ void __launch_bounds__(kWppThreads) k_force_f64(WppArgs a, const doub
         const double rhoi = (double)a.fthermo[p].x, Ai = ac[p].x, ci = ac[p].y, hinvi = hh[p].x, HHi = hh[p].y;
         const double normi = kNorm * hinvi * hinvi * hinvi * hinvi;
         const float Ti = vi.w * B.Hs, Ti2 = Ti * Ti * kF64Margin;
-        double Sx = 0.0, Sy = 0.0, Sz = 0.0, Su = 0.0, vsmax = 0.0;
-        int np = 0, nh = 0;
+        double Sx = 0.0, Sy = 0.0, Sz = 0.0, Su = 0.0, vsmax = 0.0;   // sums: at most eight terms
+        F64Sum4 Q;   // of the earlier ones
+        int np = 0, nh = 0, nev = 0;
         unsigned long long hs = 0;
         // the pair terms of buffered partners, one per lane
         auto eval = [&](int k) {
@@ -298,6 +363,7 @@ __global__ void __launch_bounds__(kWppThreads) k_force_f64(WppArgs a, const doub
                 __syncwarp();
                 if (nh >= 32) {
                     eval(32);
+                    if ((++nev & 7) == 0) Q.add(Sx, Sy, Sz, Su);
                     nh -= 32;
                     const int v = (int)lane < nh ? sm.j[lane + 32] : 0;
                     __syncwarp();
@@ -310,7 +376,12 @@ __global__ void __launch_bounds__(kWppThreads) k_force_f64(WppArgs a, const doub
         scan();
         eval(nh);
         __syncwarp();
-        f64_fold4(Sx, Sy, Sz, Su);
+        if (nev >= 8) {
+            Q.add(Sx, Sy, Sz, Su);
+            Q.fold(Sx, Sy, Sz, Su);
+        } else {
+            f64_fold4(Sx, Sy, Sz, Su);
+        }
         vsmax = warp_max(vsmax);
         np = warp_sum(np);
         if (HASH) hs = warp_sum(hs);

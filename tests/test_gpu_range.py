@@ -1,12 +1,13 @@
-"""Results at the ends of the FP32 range: boxes, conductivities and densities
-whose intermediate values leave the normal numbers or pass any fixed constant."""
+"""Results at the ends of a format's range: boxes, conductivities and densities
+whose intermediate values leave the normal numbers or pass any fixed constant,
+and sums whose terms cancel to the last bits."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 import workloads as W
-from sph_cases import as_f32, check_force, dev, gpu_density, gpu_grid, host, oracle_all
+from sph_cases import as_f32, check_force, dev, gpu_density, gpu_force, gpu_grid, host, oracle_all
 
 pytestmark = pytest.mark.gpu
 
@@ -109,3 +110,28 @@ def test_gravity_of_close_pairs_in_a_small_box(S, ctx, soft, units):
     assert np.array_equal(host(nn), o["n_nodes"]) and np.array_equal(host(npr), o["n_pairs"])
     err = np.linalg.norm(host(acc) - o["acc"], axis=1)
     assert np.all(err <= 2e-5 * o["scale"]), (err / o["scale"]).max()
+
+
+def test_fp64_force_of_mirrored_partners(S, ctx):
+    """Fourteen pairs of equal partners on opposite sides of a particle, whose
+    terms cancel, and one of mass 2^-40: the sum is its term, which rounding
+    the others' sums to 2^-53 of them would bury (their magnitudes are about
+    2^40 times it). One term per lane: only the fold over the lanes adds."""
+    rng = np.random.default_rng(23)
+    o = rng.integers(-60_000, 60_000, (14, 3)) * 2.0 ** -20
+    lone = np.array([[31_007, -20_011, 9_001]]) * 2.0 ** -20
+    pos = np.concatenate([np.zeros((1, 3)), o, -o, lone]) + 0.5
+    n = len(pos)
+    mass = np.ones(n)
+    mass[-1] = 2.0 ** -40
+    h = np.full(n, 0.15, np.float32)
+    one = np.ones(n, np.float32)
+    p = W.Particles(pos, np.zeros((n, 3)), mass, np.ones(n), 1.0)
+    params = S.default_params(flags=S.SPH_FP64)
+    g = gpu_force(S, ctx, gpu_grid(S, ctx, p, params), p, h, one, one, params)
+    assert g["rc"] == 0
+    H, r = float(h[0]), np.linalg.norm(lone[0])
+    a, b = max(1 - r / H, 0.0), max(0.5 - r / H, 0.0)
+    F = 8 / np.pi * H ** -4 * (24 * b * b - 6 * a * a) / r
+    want = mass[-1] * 2 * (params.gamma - 1.0) * F * lone[0]
+    assert np.all(np.abs(g["acc"][0] - want) <= 2.0 ** -22 * np.abs(want))
