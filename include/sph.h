@@ -454,11 +454,12 @@ sph_status sph_gravity(sph_ctx *ctx, const sph_grid *grid, const int32_t *active
  * writes dL/dx (g_pos, n x 3), dL/du (g_u, n) and dL/dm (g_mass, n) through
  * the whole chain: the implicit dependence of h on the positions
  * (dh/dx = -(dN/dx)/(dN/dh)), rho and d rho/dh, the grad-h factor Omega, the
- * pressure and viscosity terms. Velocities are constants. The pair sets come
- * from the neighbour lists of the last sph_density call on the grid, if it
- * recorded them for every particle and each position and h is the one they were
- * made with (checked on the device); otherwise, and for particles whose list
- * did not fit, from walking the grid. FP32 pair terms with compensated sums;
+ * pressure and viscosity terms. Velocities are constants. A particle's pair set
+ * comes from its neighbour list if the last sph_density call on the grid recorded
+ * one (every particle's in an all-active call, the active ones' with
+ * SPH_PARTIAL_LISTS) and every position and h is the one the lists were made with
+ * (checked on the device); otherwise, and where a list did not fit, from walking
+ * the grid. FP32 pair terms with compensated sums;
  * deterministic (gathers). The first call on a grid allocates its adjoint
  * workspace (~64 bytes/particle).
  */
