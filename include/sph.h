@@ -19,9 +19,8 @@
  *
  * Errors: every call validates its arguments on the host and returns a
  * status synchronously; kernels run asynchronously on `stream`. Conditions
- * found on the device (non-convergence, h >= L/2, non-finite input, a bounded
- * wait that ran out) set bits in a device status word that sph_sync_status()
- * returns. Nothing here traps or aborts; no exception crosses the ABI.
+ * found on the device (non-convergence, h >= L/2, non-finite input) set bits in
+ * a device status word that sph_sync_status() returns. Nothing here traps or aborts; no exception crosses the ABI.
  * sph_last_error() holds a message for the last non-OK status.
  */
 #ifndef SPH_GB300_H
@@ -39,7 +38,7 @@ typedef enum {
     SPH_ERR_CUDA = 2,           /* a CUDA runtime call failed; see sph_last_error() */
     SPH_ERR_NOT_CONVERGED = 3,  /* some h did not converge within max_iter (device) */
     SPH_ERR_H_TOO_LARGE = 4,    /* some h would reach L/2 (minimum image breaks) (device) */
-    SPH_ERR_TIMEOUT = 5,        /* a bounded device-side wait ran out (device) */
+    SPH_ERR_TIMEOUT = 5,        /* reserved: no wait that runs out changes a result */
     SPH_ERR_OOM = 6             /* device allocation failed */
 } sph_status;
 
@@ -78,7 +77,7 @@ typedef enum {
 /* Device status bits returned in sph_stats.status */
 #define SPH_ST_NOT_CONVERGED 0x01
 #define SPH_ST_H_TOO_LARGE   0x02
-#define SPH_ST_TIMEOUT       0x04
+#define SPH_ST_TIMEOUT       0x04  /* reserved, see SPH_ERR_TIMEOUT */
 #define SPH_ST_INVALID       0x08
 
 typedef struct sph_ctx sph_ctx;    /* opaque, library-owned */
@@ -461,7 +460,7 @@ sph_status sph_gravity(sph_ctx *ctx, const sph_grid *grid, const int32_t *active
  * (checked on the device); otherwise, and where a list did not fit, from walking
  * the grid. FP32 pair terms with compensated sums;
  * deterministic (gathers). The first call on a grid allocates its adjoint
- * workspace (~64 bytes/particle).
+ * workspace (72 bytes/particle).
  */
 sph_status sph_backward(sph_ctx *ctx, const sph_grid *grid, const float *vel, const float *u,
                         const float *h, const float *rho, const float *omega, const float *g_acc,

@@ -411,7 +411,7 @@ sph_status sph_backward(sph_ctx* ctx, const sph_grid* grid, const float* vel, co
     sph_status st = check_params(ctx, params);
     if (st) return st;
     if (params->flags & (SPH_FP64 | SPH_PLAIN_FP32 | SPH_WARP_GROUP))
-        return fail(ctx, SPH_ERR_INVALID, "sph_backward runs the FP32 thread path only");
+        return fail(ctx, SPH_ERR_INVALID, "sph_backward runs in FP32, on the default path");
     if (cudaSetDevice(ctx->device)) return fail(ctx, SPH_ERR_CUDA, "cudaSetDevice failed");
     BackwardLaunch b;
     b.vel = vel;

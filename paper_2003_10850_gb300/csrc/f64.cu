@@ -29,7 +29,7 @@ constexpr float kF64Margin = 1.f + 1.9073486328125e-06f;   // 2^-19: FP32 square
 struct F64Smem {
     WppSmem w;
     double r[kF64Near];                       // distance (box units)
-    unsigned long long d2[kF64Near];          // exact squared distance (integer units); as double after f64 prepare
+    unsigned long long d2[kF64Near];          // exact squared distance (integer units); prepare() makes it a double
     float m[kF64Near];
     int j[kF64Near];
 };

@@ -7,9 +7,10 @@
 //
 // The tree is the grid's hierarchy (a leaf is 8 consecutive Morton-sorted
 // particles, a node 8 consecutive nodes of the level below). Its node boxes are
-// exact integer boxes, so every decision of the walk is taken in exact integer
-// arithmetic on coarse coordinates (integer coordinates >> 8), with no
-// FP64 on the per-node or per-pair path:
+// exact integer boxes, and the rule of the walk is one of exact integer arithmetic
+// on coarse coordinates (integer coordinates >> 8); FP32 tests with a margin decide
+// where they are sure of its outcome, the rule itself elsewhere, with no FP64 on the
+// per-node or per-pair path:
 //   D2 = sum_a G_a^2, G_a the periodic gap between X_i and the box on axis a;
 //   F2 = sum_a F_a^2, F_a the periodic distance to the far side, rounded up;
 //   L2 = l^2, l the box's largest side;  RCi = ceil((r_cut 2^24 / L)^2);

@@ -5,7 +5,7 @@
 // and the others (inactive neighbours included) are drifted to the current
 // time. These kernels are the device side of that bookkeeping:
 //   k_timebins      bin of each particle from its Courant step dt = C h / v_sig
-//   k_active_flags  which particles end a step at integer time `tick`
+//                   (which of them end a step at integer time `tick`: k_flag_list, grid.cu)
 //   k_kick          v += a dt_bin, u += du/dt dt_bin for the active particles
 //                   (optionally copying the kicked values to the predictions)
 //   k_drift         x += v dt for every particle (FP64 positions, periodic), and

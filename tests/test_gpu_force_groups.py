@@ -99,6 +99,17 @@ def test_groups_in_every_variant(S, ctx, state, grid, least, variant, switch):
                 assert np.all(np.abs(dc - co)[idx] <= 1e-4 * cs[idx] + 1e-30)
 
 
+@pytest.mark.parametrize("span", [8, 512, 4096])
+def test_groups_of_other_spans(S, ctx, state, grid, least, span):
+    """Groups confined to aligned runs of 8, 512 or 4096 sorted particles."""
+    s, p = state, state["p"]
+    f = oracle.force(s["X"], p.vel, p.mass, p.u, s["h"], s["rho"], s["om"])
+    half = W.sample_indices(p.n, least + 1500, seed=6).astype(np.int32)
+    g = gpu_force(S, ctx, grid, p, s["h"], s["rho"], s["om"], S.default_params(group_size=span), active=half)
+    assert g["rc"] == 0
+    check_force(g, f, half, 1e-4)
+
+
 def test_padded_lists_on_both_sides_of_the_rule(S, ctx, state, grid, least):
     """The host sees only the capacity (every particle); the device's count
     decides. A group tests its candidates for all of its members, the
