@@ -47,10 +47,10 @@ FP32_LANES_PER_SM = 128
 # dram__bytes_write.sum), warp instructions (smsp__inst_executed.sum), serialised durations,
 # and the member-parallel kernel's pipe utilisation; the call counted 118,572,011 density pairs
 DENSITY_NCU_2M = {"kernels": "k_density_mp + k_density_wpp", "launch": "2M clustered, 100 % sub-step",
-                  "dram_bytes": (129.718016e6 + 458.693888e6) + (72.817152e6 + 42.396928e6),
-                  "warp_inst": 3.403872364e9 + 9.68670724e8,
-                  "ms": 4.384064 + 1.612096, "density_pairs": 118_572_011,
-                  "fma_pipe_pct": 26.62, "alu_pipe_pct": 39.68, "issue_active_pct": 62.85}
+                  "dram_bytes": (131.756032e6 + 461.215232e6) + (96.443904e6 + 72.384256e6),
+                  "warp_inst": 3.229635350e9 + 9.14835824e8,
+                  "ms": 4.103840 + 1.417280, "density_pairs": 118_572_011,
+                  "fma_pipe_pct": 26.94, "alu_pipe_pct": 42.50, "issue_active_pct": 63.78}
 # DRAM bytes of one density launch per active particle, scaled by the active particles of a launch
 DENSITY_DRAM_BYTES_PER_ACTIVE = DENSITY_NCU_2M["dram_bytes"] / 2_000_000
 H_PERTURB = 0.02            # per-step log-normal scatter of the h guesses: the density change between steps

@@ -18,7 +18,7 @@
 // sum over plain sums of leaves 0.6.
 // One particle per thread, every candidate tested and every square root and
 // division taken in FP64 in the pair loop, took 2.9 + 3.1 ms (density + force)
-// for 32,768 lattice particles; this form takes 0.71 + 0.54 ms.
+// for 32,768 lattice particles; this form takes 0.73 + 0.58 ms.
 #include "wpp.cuh"
 
 namespace sph {
